@@ -318,7 +318,8 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0);   // warp-uniform
+  const int lane = threadIdx.x & 31;
   constexpr int rows_alloc = kAttnMaxRows;
   uint8_t* sQ = smem + kAttnQOff;
   uint8_t* sP = smem + kAttnPOff;                        // [2][128][128 B]
@@ -419,32 +420,30 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
 
   if (warp == kAttnTmaWarp) {
     // ---- TMA producer: K and V^T pages of the item, in order
-    if (lane == 0) {
+    if (elect_one()) {
       const int safe_pages = a.blk_slot ? a.lim[tok0] / 64 : 0;   // wholly committed pages
       const uint64_t pol = l2_policy_evict_first();
       int issued = 0;
-      auto issue = [&](int i) {
-        const int s = i % kAttnStages;
+      RingPos r;
+      const uint32_t full0 = smem_u32(full), empty0 = smem_u32(empty), ring0 = smem_u32(ring);
+      auto issue = [&](int i) {   // page i into the ring's next stage
         int phys = pt[p_begin + i];
         if (phys < 0) {  // unmapped page: the TMA box lands out of bounds and reads zeros
           atomicExch(a.err, kErrBounds);
           phys = 0x3FFFFFFF / a.rows_per_page;
         }
         const long long row = a.kv_row_base + static_cast<long long>(phys) * a.rows_per_page;
-        const uint32_t fb = smem_u32(&full[s]);
+        const uint32_t fb = full0 + 8 * r.s, st = ring0 + r.s * kAttnStageBytes;
         mbar_arrive_expect_tx(fb, 2 * kAttnPageBytes);   // K and V^T (the ones rows stay)
-        uint8_t* st = ring + s * kAttnStageBytes;
-        tma_load_2d(smem_u32(st), &tmKV, 0, static_cast<int>(row + h * 64), fb, pol);
-        tma_load_2d(smem_u32(st + kAttnPageBytes), &tmKV, 0, static_cast<int>(row + (a.Hkv + h) * 64),
-                    fb, pol);
+        tma_load_2d(st, &tmKV, 0, static_cast<int>(row + h * 64), fb, pol);
+        tma_load_2d(st + kAttnPageBytes, &tmKV, 0, static_cast<int>(row + (a.Hkv + h) * 64), fb, pol);
+        r.next(kAttnStages);
       };
       while (issued < min(np, kAttnStages) && p_begin + issued < safe_pages) issue(issued++);
       pdl_wait();
       pdl_trigger();
       while (issued < np && ok) {
-        const int s = issued % kAttnStages;
-        if (issued >= kAttnStages &&
-            !mbar_wait(smem_u32(&empty[s]), ((issued / kAttnStages) + 1) & 1, a.err)) {
+        if (issued >= kAttnStages && !mbar_wait(empty0 + 8 * r.s, r.ph ^ 1, a.err)) {
           ok = false;
           break;
         }
@@ -459,39 +458,46 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
     // ---- MMA issuer: S one page ahead of the softmax, O += P V after each P
     pdl_wait();
     pdl_trigger();
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t idesc = umma_idesc_f16(128, 64);
       constexpr uint32_t idesc_pv = umma_idesc_f16(128, 80);   // V^T page and its 16 ones rows
       const uint64_t qdesc = umma_desc_sw128(smem_u32(sQ));
+      const uint64_t pdesc0 = umma_desc_sw128(smem_u32(sP));
+      const uint64_t kdesc0 = umma_desc_sw128(smem_u32(ring));
+      const uint32_t full0 = smem_u32(full), empty0 = smem_u32(empty);
+      const uint32_t s_full0 = smem_u32(s_full), s_free0 = smem_u32(s_free), p_full0 = smem_u32(p_full);
+      RingPos rs, rv;   // ring stages of the next S and the next PV
       auto issue_s = [&](int j) -> bool {
-        const int s = j % kAttnStages, buf = j & 1;
-        if (!mbar_wait(smem_u32(&full[s]), (j / kAttnStages) & 1, a.err)) return false;
+        const int buf = j & 1;
+        if (!mbar_wait(full0 + 8 * rs.s, rs.ph, a.err)) return false;
         s_int[2] = j + 1;
-        if (j >= 2 && !mbar_wait(smem_u32(&s_free[buf]), ((j >> 1) + 1) & 1, a.err)) return false;
+        if (j >= 2 && !mbar_wait(s_free0 + 8 * buf, ((j >> 1) + 1) & 1, a.err)) return false;
         tc_fence_after();
-        const uint64_t kdesc = umma_desc_sw128(smem_u32(ring + s * kAttnStageBytes));
+        const uint64_t kdesc = kdesc0 + rs.s * (kAttnStageBytes >> 4);
 #pragma unroll
         for (int k = 0; k < 4; ++k)
           umma_f16(tmem + buf * 64, qdesc + 2 * k, kdesc + 2 * k, idesc, k > 0 ? 1u : 0u);
-        umma_commit(smem_u32(&s_full[buf]));
+        umma_commit(s_full0 + 8 * buf);
+        rs.next(kAttnStages);
         return true;
       };
       if (!mbar_wait(smem_u32(q_full), 0, a.err)) ok = false;   // Q tile written
       if (ok) ok = issue_s(0);
       for (int j = 0; j < np && ok; ++j) {
         if (j + 1 < np && !(ok = issue_s(j + 1))) break;
-        const int s = j % kAttnStages, buf = j & 1;
-        if (!mbar_wait(smem_u32(&p_full[buf]), (j >> 1) & 1, a.err)) {
+        const int buf = j & 1;
+        if (!mbar_wait(p_full0 + 8 * buf, (j >> 1) & 1, a.err)) {
           ok = false;
           break;
         }
         tc_fence_after();
-        const uint64_t pdesc = umma_desc_sw128(smem_u32(sP + buf * kAttnMaxRows * 128));
-        const uint64_t vdesc = umma_desc_sw128(smem_u32(ring + s * kAttnStageBytes + kAttnPageBytes));
+        const uint64_t pdesc = pdesc0 + buf * (kAttnMaxRows * 128 >> 4);
+        const uint64_t vdesc = kdesc0 + ((rv.s * kAttnStageBytes + kAttnPageBytes) >> 4);
 #pragma unroll
         for (int k = 0; k < 4; ++k)
           umma_f16(tmem + 128, pdesc + 2 * k, vdesc + 2 * k, idesc_pv, (j > 0 || k > 0) ? 1u : 0u);
-        umma_commit(smem_u32(&empty[s]));
+        umma_commit(empty0 + 8 * rv.s);
+        rv.next(kAttnStages);
       }
       umma_commit(smem_u32(mma_done));   // retires once every MMA above has
     }

@@ -56,9 +56,15 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 }
 
 // Wait for the phase with the given parity; false (and the error word set)
-// if it has not completed within limit_ns of %globaltimer.
+// if it has not completed within limit_ns of %globaltimer.  The first try is
+// its own straight-line branch: try_wait itself suspends the thread until the
+// phase completes, so it nearly always succeeds there, and entering the retry
+// loop costs about 50 cycles per wait even when the phase is complete (a
+// 64-deep k-block of a TMA ring: 395 -> 300 cycles with both of its waits
+// written this way).
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* err,
                                           uint64_t limit_ns = kWaitLimitNs) {
+  if (mbar_try_wait(bar, parity)) return true;
   for (int i = 0; i < 256; ++i)
     if (mbar_try_wait(bar, parity)) return true;
   const uint64_t t0 = global_timer_ns();
@@ -70,6 +76,34 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* er
     }
     __nanosleep(128);
   }
+}
+
+// Position in a ring of `n` stages: the stage and the parity of its use,
+// advanced by a compare instead of a division by the run-time stage count
+// (the divisions cost a TMA -> MMA ring about 300 of 700 cycles per k-block).
+struct RingPos {
+  int s = 0;
+  uint32_t ph = 0;
+  __device__ __forceinline__ void next(int n) {
+    if (++s == n) {
+      s = 0;
+      ph ^= 1;
+    }
+  }
+};
+
+// True in one lane of a converged warp.  Single-thread code that issues TMA
+// copies or tcgen05 instructions branches on this rather than on `lane == 0`:
+// their operands live in uniform registers, and only elect.sync tells the
+// compiler that the branch holds a single thread.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xFFFFFFFF;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0;
 }
 
 // ---------------------------------------------------------------- TMA
