@@ -24,10 +24,11 @@
 // The max only moves when a page raises it by more than 2^8: then the thread
 // first rescales its O row in TMEM (and l with it) by exp2(m_old - m_new).  Smaller
 // rises keep the old m, so P stays <= 2^8 (well inside fp16).  Either way
-// O / l is the softmax-weighted sum.  Warps 0-3 own rows 0-127 (TMEM lanes;
-// warps whose rows are all padding only keep the barriers' pace); warp 4
-// streams K/V pages by TMA (128-byte swizzle) through a ring of stages; warp
-// 5 issues the MMAs, S one page ahead of the softmax, S double-buffered.
+// O / l is the softmax-weighted sum.  Block row rr sits in MMA row (TMEM lane)
+// 32 (rr mod 4) + rr / 4, so warps 0-3 (one lane quarter each) hold a quarter
+// of the rows each, whatever their number; warp 4 streams K/V pages by TMA
+// (128-byte swizzle) through a ring of stages; warp 5 issues the MMAs, S one
+// page ahead of the softmax, S double-buffered.
 //
 // Merge over items, item order 0, 1, ...: M = max m_i, w_i = exp2(m_i - M),
 // coef_i = w_i / sum_j w_j l_j, O = sum coef_i O_i.  A block with one item
@@ -62,6 +63,7 @@ constexpr int kAttnSoftThreads = kAttnSoftWarps * 32;
 constexpr int kAttnThreads = kAttnSoftThreads + 64;   // + TMA warp, MMA warp
 constexpr int kAttnTmaWarp = kAttnSoftWarps, kAttnMmaWarp = kAttnSoftWarps + 1;
 constexpr int kAttnTmemCols = 256;        // S[2] at columns 0, 64; O at 128
+constexpr int kAttnPtAhead = 64;         // page numbers an item reads up front
 constexpr float kAttnRescale = 8.0f;      // log2 growth of the max that forces a rescale
 constexpr int kAttnRingBytes = kAttnStages * kAttnStageBytes;
 // Q [128][128 B] | P[2] [128][128 B] | ring | barriers.  After the pages are
@@ -71,7 +73,7 @@ constexpr int kAttnQOff = 0;
 constexpr int kAttnPOff = kAttnMaxRows * 128;
 constexpr int kAttnRingOff = kAttnPOff + 2 * kAttnMaxRows * 128;
 constexpr int kAttnBarOff = kAttnRingOff + kAttnRingBytes;
-constexpr int kAttnSmemBytes = 1024 + kAttnBarOff + 256 + 2 * kAttnSoftThreads * 4;
+constexpr int kAttnSmemBytes = 1024 + kAttnBarOff + 256 + kAttnMaxRows * 4 + kAttnPtAhead * 4;
 constexpr int kAttnRowsFloats = (kAttnMaxRows + kAttnMaxCluster) * kAttnRow;
 static_assert(kAttnRingOff >= kAttnRowsFloats * 4 && kAttnRingBytes >= kAttnRowsFloats * 4,
               "Q + P hold the owner-grouped rows, the ring the received rows");
@@ -109,24 +111,49 @@ __device__ __forceinline__ uint32_t sw128(int row, int chunk) {
   return static_cast<uint32_t>(row * 128 + ((chunk ^ (row & 7)) << 4));
 }
 
-__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t (&r)[16]) {
+// 16 TMEM lanes x 64 (x8) or 8 (x1) fp32 columns, in the 16x256b fragment
+// layout: thread t receives, for column group j (8 columns), r[4 j + 2 q + e] =
+// lane t / 4 + 8 q, column 8 j + 2 (t mod 4) + e.  A row is spread over four
+// neighbouring threads.
+__device__ __forceinline__ void tmem_ld_16x256b_x8(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      "tcgen05.ld.sync.aligned.16x256b.x8.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
         "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15])
+        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
+        "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
+        "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_st_16x256b_x8(uint32_t taddr, const uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.16x256b.x8.b32 [%0], "
+      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
+      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(taddr),
+      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
+      "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]),
+      "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]),
+      "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]),
+      "r"(r[29]), "r"(r[30]), "r"(r[31])
+      : "memory");
+}
+__device__ __forceinline__ void tmem_ld_16x256b_x1(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_st_16x256b_x1(uint32_t taddr, const uint32_t (&r)[4]) {
+  asm volatile("tcgen05.st.sync.aligned.16x256b.x1.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr),
+               "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3])
+               : "memory");
 }
 
 __device__ __forceinline__ uint32_t tmem_ld1(uint32_t taddr) {
   uint32_t r;
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr));
   return r;
-}
-
-__device__ __forceinline__ void tmem_st1(uint32_t taddr, uint32_t v) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(taddr), "r"(v) : "memory");
 }
 
 // 2^x on the SFU (PTX ex2.approx.ftz.f32, one instruction): the P values are
@@ -149,166 +176,161 @@ struct AttnSync {
   uint64_t *s_full, *s_free, *p_full;
   uint64_t* empty;   // [stages] O += P V of the stage's page retired
   uint8_t* sP;       // [2][128][128 B]
-  float* red;        // [128] per-thread page maxima (exchanged only when a max rises)
+  float* m_row;      // [128] per MMA row: the final running max
 };
 
-// Named barriers of the softmax warps (barrier 0 is __syncthreads).
-constexpr int kAttnBarVote = 1, kAttnBarMax = 2;
+// MMA row (TMEM lane) -> block row, and back.
+__device__ __forceinline__ int attn_block_row(int mrow) { return (mrow & 31) * 4 + (mrow >> 5); }
 
-// OR of a predicate over the softmax threads: one hardware barrier.
-__device__ __forceinline__ bool softmax_vote_or(bool v) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.ne.u32 q, %1, 0;\n\t"
-      "bar.red.or.pred p, %2, %3, q;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(r)
-      : "r"(v ? 1u : 0u), "n"(kAttnBarVote), "n"(kAttnSoftThreads)
-      : "memory");
-  return r != 0;
-}
-
-__device__ __forceinline__ void softmax_bar_max() {
-  asm volatile("bar.sync %0, %1;" ::"n"(kAttnBarMax), "n"(kAttnSoftThreads) : "memory");
-}
-
-// Online softmax over the item's pages, one thread per TMEM lane.  DUP copies
-// of each block row sit in the MMA's 128 rows (copy k of row rr at MMA row
-// k * 128 / DUP + rr, so every lane quarter -- and every SM sub-partition --
-// holds rows); the thread of copy k takes the NC = 64 / DUP columns
-// [k NC, (k + 1) NC) of every page.  Per page: S from TMEM, mask and scale,
-// this thread's maximum; the row's running max m (log2 units) only moves when
-// a page raises it by more than 2^8, so one vote over the softmax threads (a
-// hardware barrier) decides whether any row of the block rises, and only then
-// are the copies' page maxima exchanged through shared memory (always on the
-// first page, rarely after).  A rise rescales O and the row sum in O's column
-// 64 (the copy-0 thread of the row; the previous O += P V must have retired);
-// then P_j = exp2(s - m) as fp16 into row rr of the P tile.  m, P and the
-// rescale are the same for every DUP.  Waits are bounded; a warp whose wait ran out keeps passing the named
-// barriers and arriving on the MMA warp's barriers to the last page, so no
-// thread is left at a barrier.  Returns false if a wait ran out.
-template <int DUP>
+// Online softmax over the item's pages, for a warp whose lane quarter holds at
+// most 8 NSET rows.  S comes from TMEM in the 16x256b layout, so a row is
+// spread over four neighbouring threads and set q (rows 8 q .. 8 q + 7 of the
+// quarter) costs a thread 16 columns, whatever the number of rows in the block
+// is: 34 rows (a 17-token window, GQA 2) cost 16 or 32 exponentials per thread
+// and page.  Per page: S, mask and scale, the row's maximum (two shuffles);
+// the row's running max m (log2 units) only moves when a page raises it by
+// more than 2^8 (always on the first page, rarely after).  A rise rescales O
+// and the row sum in O's column 64 (the previous O += P V must have retired);
+// then P_j = exp2(s - m) as fp16 into the P tile.  No step of a page needs
+// another warp: the warps meet only on the MMA warp's barriers.  Bound by the
+// serial chain of a page (TMEM load, max, exponentials, P store, fence).
+// Waits are bounded; a warp whose wait ran out keeps arriving on the MMA
+// warp's barriers to the last page.  Returns false if a wait ran out.
+template <int NSET>
 __device__ __forceinline__ bool attn_softmax(const AttnArgs& a, const AttnSync& y, uint32_t tmem,
-                                             int np, int p_begin, int R, int tok0, float& m) {
-  constexpr int RPC = kAttnMaxRows / DUP;   // MMA rows per copy
-  constexpr int NC = 64 / DUP;              // columns per thread
-  constexpr int NCH = NC / 8;               // 8-column chunks per thread
-  const int mrow = threadIdx.x, warp = mrow >> 5, lane = mrow & 31;   // MMA row = TMEM lane
-  const int cp = mrow / RPC, rr = mrow % RPC;
-  const int col0 = cp * NC;
-  const bool busy = ((warp * 32) % RPC) < R;   // the warp holds at least one real row
-  const int lim_r = rr < R ? a.lim[tok0 + rr / a.G] : -1;
+                                             int warp, int np, int p_begin, int R, int tok0) {
+  constexpr int NH = (NSET + 1) / 2;   // 16-lane halves of the quarter
+  const int lane = threadIdx.x & 31;
+  const int quad = lane & 3;
+  float m[NSET];
+  int lim[NSET];
+  int full_lim = 0x7FFFFFFF;   // every row of the warp sees the keys up to here
+#pragma unroll
+  for (int q = 0; q < NSET; ++q) {
+    const int rr = (8 * q + (lane >> 2)) * 4 + warp;
+    m[q] = -INFINITY;
+    lim[q] = rr < R ? a.lim[tok0 + rr / a.G] : -1;
+    if (rr < R) full_lim = min(full_lim, lim[q]);
+  }
+  full_lim = __reduce_min_sync(0xFFFFFFFFu, full_lim);
   const uint32_t trow = tmem + (static_cast<uint32_t>(warp * 32) << 16);
+  // row (warp * 32 + lane / 4) of the P tile; chunk j of row r sits at (j ^ (r & 7)) * 16
+  const uint32_t p0 = smem_u32(y.sP) + (warp * 32 + (lane >> 2)) * 128 + ((lane >> 2) << 4) + 4 * quad;
+  const uint32_t s_full0 = smem_u32(y.s_full), s_free0 = smem_u32(y.s_free), p_full0 = smem_u32(y.p_full);
   const float kScaleLog2 = 0.125f * 1.4426950408889634f;   // 1/sqrt(64) in log2 units
   bool ok = true;
   // waits are warp-uniform; after a failure the warp stops waiting
-  auto wwait = [&](uint64_t* bar, uint32_t parity) {
-    if (ok) ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(bar), parity, a.err)) != 0;
+  auto wwait = [&](uint32_t bar, uint32_t parity) {
+    if (ok) ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, a.err)) != 0;
     return ok;
   };
   for (int j = 0; j < np; ++j) {
     const int buf = j & 1;
-    const bool have = wwait(&y.s_full[buf], (j >> 1) & 1) && busy;
-    // 1. this thread's columns of S_j; the buffer is free once every warp has read
-    float sv[NC];
-    float pm = -INFINITY;
+    const bool have = wwait(s_full0 + 8 * buf, (j >> 1) & 1);
+    // 1. S_j; the buffer is free once every warp has read it
+    uint32_t sr[NH][32];
     if (have) {
       tc_fence_after();
-      uint32_t sr[NC];
-      if constexpr (NC == 16) {
-        tmem_ld16_nowait(trow + buf * 64 + col0, *reinterpret_cast<uint32_t(*)[16]>(sr));
-      } else if constexpr (NC == 32) {
-        tmem_ld32_nowait(trow + buf * 64 + col0, *reinterpret_cast<uint32_t(*)[32]>(sr));
-      } else {
-        tmem_ld32_nowait(trow + buf * 64, *reinterpret_cast<uint32_t(*)[32]>(sr));
-        tmem_ld32_nowait(trow + buf * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(sr + 32));
-      }
+#pragma unroll
+      for (int hf = 0; hf < NH; ++hf)
+        tmem_ld_16x256b_x8(trow + (static_cast<uint32_t>(16 * hf) << 16) + buf * 64, sr[hf]);
       tmem_wait_ld();
-      // 2. mask (keys past the row's limit: only on the window's last pages),
-      //    this thread's maximum (of the unscaled scores; the scale is positive)
-      const int key0 = (p_begin + j) * 64 + col0;
-      if (__all_sync(0xFFFFFFFFu, rr >= R || key0 + NC - 1 <= lim_r)) {
-#pragma unroll
-        for (int k = 0; k < NC; ++k) sv[k] = __uint_as_float(sr[k]);
-      } else {
-#pragma unroll
-        for (int k = 0; k < NC; ++k) sv[k] = key0 + k <= lim_r ? __uint_as_float(sr[k]) : -INFINITY;
-      }
-      // max as a tree of three-way maxima (a chain of NC dependent fmax
-      // would dominate the page)
-      float mt[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        mt[e] = sv[e];
-        int k = e + 8;
-#pragma unroll
-        for (; k + 8 < NC; k += 16) mt[e] = fmax3(mt[e], sv[k], sv[k + 8]);
-        if (k < NC) mt[e] = fmaxf(mt[e], sv[k]);
-      }
-      pm = fmax3(fmax3(mt[0], mt[1], mt[2]), fmax3(mt[3], mt[4], mt[5]), fmaxf(mt[6], mt[7])) *
-           kScaleLog2;
     }
     tc_fence_before();
     __syncwarp();
-    if (lane == 0) mbar_arrive(smem_u32(&y.s_free[buf]));
-    // 3. does any row rise by more than 2^8?  Then the row's page max over its
-    //    DUP copies (copy k at MMA row k * RPC + rr).
-    const bool any = softmax_vote_or(pm > m + kAttnRescale);
-    float mx = -INFINITY;
-    if (any) {
-      y.red[mrow] = pm;
-      softmax_bar_max();
-#pragma unroll
-      for (int k = 0; k < DUP; ++k) mx = fmaxf(mx, y.red[k * RPC + rr]);
-    }
-    // 4. a rise rescales O and the row sum first.  tcgen05.ld / st are
-    //    warp-collective: a warp with any rising row rescales all its rows,
-    //    the others by exactly 1.
-    const bool rise = any && mx > m + kAttnRescale;
-    const float alpha = !rise ? 1.f : ((m == -INFINITY) ? 0.f : exp2f(m - mx));
-    if (cp == 0 && j > 0 && __any_sync(0xFFFFFFFFu, rise) &&
-        wwait(&y.empty[(j - 1) % kAttnStages], ((j - 1) / kAttnStages) & 1)) {
-      tc_fence_after();
-#pragma unroll
-      for (int hh = 0; hh < 2; ++hh) {
-        uint32_t o32[32];
-        tmem_ld32_nowait(trow + 128 + hh * 32, o32);
-        tmem_wait_ld();
-#pragma unroll
-        for (int k = 0; k < 32; ++k) o32[k] = __float_as_uint(alpha * __uint_as_float(o32[k]));
-        tmem_st32(trow + 128 + hh * 32, o32);
-      }
-      // and the row sum, O's column 64
-      const uint32_t l1 = tmem_ld1(trow + 192);
-      tmem_wait_ld();
-      tmem_st1(trow + 192, __float_as_uint(alpha * __uint_as_float(l1)));
-      tmem_wait_st();
-    }
-    if (rise) m = mx;
-    // 5. P_j = exp2(s - m) (fp16) into row rr of the P tile
+    if (lane == 0) mbar_arrive(s_free0 + 8 * buf);
     if (have) {
-      const float sub = (m == -INFINITY) ? 0.f : m;
-      uint8_t* prow = y.sP + buf * kAttnMaxRows * 128;
+      // 2. mask: keys past the row's limit (only on a window's last pages)
+      const int key0 = (p_begin + j) * 64;
+      if (key0 + 63 > full_lim) {
 #pragma unroll
-      for (int c = 0; c < NCH; ++c) {
-        float p[8];
+        for (int q = 0; q < NSET; ++q)
 #pragma unroll
-        for (int e = 0; e < 8; ++e) p[e] = ex2_sfu(fmaf(sv[8 * c + e], kScaleLog2, -sub));
-        uint32_t w4[4];
+          for (int k = 0; k < 16; ++k) {
+            const int key = key0 + 8 * (k >> 1) + 2 * quad + (k & 1);
+            uint32_t& v = sr[q >> 1][4 * (k >> 1) + 2 * (q & 1) + (k & 1)];
+            v = key <= lim[q] ? v : 0xFF800000u;
+          }
+      }
+      // 3. the row's page max (of the unscaled scores; the scale is positive)
+      //    over the four threads of the row; does any row rise by more than 2^8?
+      float pm[NSET];
+      bool rise[NSET], any = false;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          __half2 hv = __floats2half2_rn(p[2 * e], p[2 * e + 1]);
-          w4[e] = *reinterpret_cast<uint32_t*>(&hv);
+      for (int q = 0; q < NSET; ++q) {
+        auto S = [&](int k) {
+          return __uint_as_float(sr[q >> 1][4 * (k >> 1) + 2 * (q & 1) + (k & 1)]);
+        };
+        float t = fmax3(fmax3(S(0), S(1), S(2)), fmax3(S(3), S(4), S(5)), fmax3(S(6), S(7), S(8)));
+        t = fmax3(t, fmax3(S(9), S(10), S(11)), fmax3(S(12), S(13), fmaxf(S(14), S(15))));
+        t = fmaxf(t, __shfl_xor_sync(0xFFFFFFFFu, t, 1));
+        t = fmaxf(t, __shfl_xor_sync(0xFFFFFFFFu, t, 2));
+        pm[q] = t * kScaleLog2;
+        rise[q] = pm[q] > m[q] + kAttnRescale;
+        any |= rise[q];
+      }
+      // 4. a rise rescales O and the row sum first.  tcgen05.ld / st are
+      //    warp-collective: a warp with any rising row rescales all its rows,
+      //    the others by exactly 1.
+      if (__any_sync(0xFFFFFFFFu, any)) {
+        float alpha[2 * NH];
+#pragma unroll
+        for (int q = 0; q < 2 * NH; ++q) {
+          alpha[q] = 1.f;
+          if (q < NSET) {
+            const int qq = q < NSET ? q : 0;
+            if (rise[qq]) {
+              alpha[q] = m[qq] == -INFINITY ? 0.f : exp2f(m[qq] - pm[qq]);
+              m[qq] = pm[qq];
+            }
+          }
         }
-        *reinterpret_cast<uint4*>(prow + sw128(rr, col0 / 8 + c)) =
-            make_uint4(w4[0], w4[1], w4[2], w4[3]);
+        if (j > 0 && wwait(smem_u32(&y.empty[(j - 1) % kAttnStages]), ((j - 1) / kAttnStages) & 1)) {
+          tc_fence_after();
+#pragma unroll
+          for (int hf = 0; hf < NH; ++hf) {
+            const uint32_t o = trow + (static_cast<uint32_t>(16 * hf) << 16) + 128;
+            uint32_t v[32], l4[4];
+            tmem_ld_16x256b_x8(o, v);
+            tmem_ld_16x256b_x1(o + 64, l4);   // the row sums, O's columns 64..71
+            tmem_wait_ld();
+#pragma unroll
+            for (int k = 0; k < 32; ++k)
+              v[k] = __float_as_uint(alpha[2 * hf + ((k >> 1) & 1)] * __uint_as_float(v[k]));
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              l4[k] = __float_as_uint(alpha[2 * hf + (k >> 1)] * __uint_as_float(l4[k]));
+            tmem_st_16x256b_x8(o, v);
+            tmem_st_16x256b_x1(o + 64, l4);
+          }
+          tmem_wait_st();
+        }
+      }
+      // 5. P_j = exp2(s - m) (fp16) into the rows of the P tile
+#pragma unroll
+      for (int q = 0; q < NSET; ++q) {
+        const float sub = (m[q] == -INFINITY) ? 0.f : m[q];
+        const uint32_t prow = p0 + buf * (kAttnMaxRows * 128) + q * (8 * 128);
+#pragma unroll
+        for (int jj = 0; jj < 8; ++jj) {
+          const int k = 4 * jj + 2 * (q & 1);
+          const float x0 = ex2_sfu(fmaf(__uint_as_float(sr[q >> 1][k]), kScaleLog2, -sub));
+          const float x1 = ex2_sfu(fmaf(__uint_as_float(sr[q >> 1][k + 1]), kScaleLog2, -sub));
+          const __half2 hv = __floats2half2_rn(x0, x1);
+          asm volatile("st.shared.b32 [%0], %1;" ::"r"(prow ^ (jj << 4)),
+                       "r"(*reinterpret_cast<const uint32_t*>(&hv))
+                       : "memory");
+        }
       }
       fence_proxy_async_smem();
     }
     tc_fence_before();
     __syncwarp();
-    if (lane == 0) mbar_arrive(smem_u32(&y.p_full[buf]));
+    if (lane == 0) mbar_arrive(p_full0 + 8 * buf);
+  }
+  if (quad == 0) {
+#pragma unroll
+    for (int q = 0; q < NSET; ++q) y.m_row[warp * 32 + 8 * q + (lane >> 2)] = m[q];
   }
   return ok;
 }
@@ -334,8 +356,11 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
   uint64_t* recv_bar = s_full + 8;
   uint64_t* q_full = s_full + 9;                         // Q tile in smem (4 warp arrivals)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_full + 12);
-  // [0] max limit, [1] last-item flag, [2] pages the MMA warp took, [3] pages issued
+  // [0] max limit, [1] last-item flag, [2] pages the MMA warp took, [3] pages
+  // issued, [4] sequence active, [5] page-table row
   int* s_int = reinterpret_cast<int*>(s_full + 13);
+  float* m_row = reinterpret_cast<float*>(s_int + 8);    // [128] running max per MMA row
+  int* pt_s = reinterpret_cast<int*>(m_row + kAttnMaxRows);   // the item's first page numbers
 
   const int c = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
   const int seq = b / a.n_sub, sub = b % a.n_sub;
@@ -344,90 +369,102 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
   // write: the window descriptors (key limits, block slots), the page table,
   // and cache pages wholly before the current window.  Every early exit is
   // uniform across the CTA, and across the cluster before its barrier.
-  if (a.blk_active != nullptr && a.blk_active[seq] == 0) return;
   const int tok0 = seq * a.QB + sub * a.QS;
   const int ntok = min(min(a.QS, a.QB - sub * a.QS), a.T - tok0);
   if (ntok <= 0) return;
   const int R = ntok * a.G;
-  const int slot = a.blk_slot ? a.blk_slot[seq] : a.fixed_slot;
+  const int nbusy = min(R, kAttnSoftWarps);   // softmax warps with rows
 
+  // One round of global latency: warp 0 reads the block's descriptors while
+  // the others set up barriers, TMEM and the ones rows.
   if (warp == 0) {
-    int mxl = -1;
-    for (int i = lane; i < ntok; i += 32) mxl = max(mxl, a.lim[tok0 + i]);
+    const int act = a.blk_active != nullptr ? a.blk_active[seq] : 1;
+    const int sl = a.blk_slot ? a.blk_slot[seq] : a.fixed_slot;
+    int lm[4];   // ntok <= 128
 #pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) mxl = max(mxl, __shfl_xor_sync(0xFFFFFFFFu, mxl, o));
-    if (lane == 0) s_int[0] = mxl;
-  }
-  __syncthreads();
-  const int maxlim = s_int[0];
-  const int npages_blk = maxlim / 64 + 1;
-  const int SP = a.split_pages;
-  const int nitems = (npages_blk + SP - 1) / SP;
-  if (maxlim < 0 || npages_blk > a.pt_stride || slot < 0 || nitems > a.max_items ||
-      R > kAttnMaxRows) {
-    if (threadIdx.x == 0) atomicExch(a.err, kErrBounds);
-    return;
-  }
-  if (c >= nitems && (nitems == 1 || !a.cluster)) return;
-  const bool in_cluster = a.cluster && nitems > 1;
-  if (c >= nitems) {   // idle cluster member: counts in the cluster barrier, owns nothing
-    cluster_arrive_release();
-    return;
-  }
-
-  if (threadIdx.x == 0) {
-    tma_prefetch_desc(&tmKV);
-    for (int s = 0; s < kAttnStages; ++s) {
-      mbar_init(smem_u32(&full[s]), 1);
-      mbar_init(smem_u32(&empty[s]), 1);
+    for (int q = 0; q < 4; ++q) lm[q] = lane + 32 * q < ntok ? a.lim[tok0 + lane + 32 * q] : -1;
+    const int mxl = __reduce_max_sync(0xFFFFFFFFu, max(max(lm[0], lm[1]), max(lm[2], lm[3])));
+    if (lane == 0) {
+      s_int[0] = mxl;
+      s_int[4] = act;
+      s_int[5] = sl;
     }
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(smem_u32(&s_full[i]), 1);
-      mbar_init(smem_u32(&s_free[i]), kAttnSoftWarps);   // one arrival per softmax warp
-      mbar_init(smem_u32(&p_full[i]), kAttnSoftWarps);
-    }
-    mbar_init(smem_u32(mma_done), 1);
-    mbar_init(smem_u32(q_full), kAttnSoftWarps);
-    if (in_cluster) {
+  } else if (warp == 1) {
+    if (lane == 0) {
+      for (int s = 0; s < kAttnStages; ++s) {
+        mbar_init(smem_u32(&full[s]), 1);
+        mbar_init(smem_u32(&empty[s]), 1);
+      }
+      for (int i = 0; i < 2; ++i) {
+        mbar_init(smem_u32(&s_full[i]), 1);
+        mbar_init(smem_u32(&s_free[i]), nbusy);   // one arrival per softmax warp with rows
+        mbar_init(smem_u32(&p_full[i]), nbusy);
+      }
+      mbar_init(smem_u32(mma_done), 1);
+      mbar_init(smem_u32(q_full), kAttnSoftWarps);
       mbar_init(smem_u32(recv_bar), 1);
-      // nitems sources, ceil(128 / nitems) rows each, arrive by bulk copy
-      const int rpo = (rows_alloc + nitems - 1) / nitems;
-      mbar_arrive_expect_tx(smem_u32(recv_bar), static_cast<uint32_t>(nitems * rpo * kAttnRow * 4));
+      s_int[2] = 0;
+      s_int[3] = 0;
+      fence_mbar_init();
     }
-    s_int[2] = 0;
-    s_int[3] = 0;
-    fence_mbar_init();
+  } else if (warp < kAttnSoftWarps) {
+    // the ones rows after every V^T page: O += P [V | 1] puts the row sum in O's column 64
+    for (int i = threadIdx.x - 64; i < kAttnStages * kAttnOnesBytes / 16; i += 64) {
+      const int st = i / (kAttnOnesBytes / 16), off = i % (kAttnOnesBytes / 16);
+      *reinterpret_cast<uint4*>(ring + st * kAttnStageBytes + 2 * kAttnPageBytes + off * 16) =
+          make_uint4(0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u);
+    }
+    fence_proxy_async_smem();
+  } else if (warp == kAttnTmaWarp) {
+    if (lane == 0) tma_prefetch_desc(&tmKV);
+  } else {
+    tmem_alloc(smem_u32(tmem_slot), kAttnTmemCols);
   }
-  // the ones rows after every V^T page: O += P [V | 1] puts the row sum in O's column 64
-  for (int i = threadIdx.x; i < kAttnStages * kAttnOnesBytes / 16; i += blockDim.x) {
-    const int st = i / (kAttnOnesBytes / 16), off = i % (kAttnOnesBytes / 16);
-    *reinterpret_cast<uint4*>(ring + st * kAttnStageBytes + 2 * kAttnPageBytes + off * 16) =
-        make_uint4(0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u);
-  }
-  fence_proxy_async_smem();
-  if (warp == kAttnMmaWarp) tmem_alloc(smem_u32(tmem_slot), kAttnTmemCols);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  const int maxlim = s_int[0], slot = s_int[5];
+  const int npages_blk = maxlim / 64 + 1;
+  const int SP = a.split_pages;
+  const int nitems = (npages_blk + SP - 1) / SP;
+  const bool active = s_int[4] != 0;
+  const bool bad = maxlim < 0 || npages_blk > a.pt_stride || slot < 0 || nitems > a.max_items ||
+                   R > kAttnMaxRows;
+  const bool in_cluster = a.cluster && nitems > 1;
+  if (!active || bad || c >= nitems) {
+    if (active && bad && threadIdx.x == 0) atomicExch(a.err, kErrBounds);
+    // idle cluster member: counts in the cluster barrier, owns nothing
+    if (active && !bad && in_cluster) cluster_arrive_release();
+    if (warp == kAttnMmaWarp) tmem_dealloc(tmem, kAttnTmemCols);
+    return;
+  }
+  if (in_cluster && threadIdx.x == 0) {
+    // nitems sources, ceil(128 / nitems) rows each, arrive by bulk copy (after
+    // the cluster barrier below)
+    const int rpo = (rows_alloc + nitems - 1) / nitems;
+    mbar_arrive_expect_tx(smem_u32(recv_bar), static_cast<uint32_t>(nitems * rpo * kAttnRow * 4));
+  }
 
   const int p_begin = c * SP;
   const int np = min(npages_blk, p_begin + SP) - p_begin;
   const int32_t* pt = a.page_table + static_cast<size_t>(slot) * a.pt_stride;
   bool ok = true;
-  float m = -INFINITY, l = 0.f;   // the row's running max (log2 units) and sum
-  float* red = reinterpret_cast<float*>(s_int + 8);        // [softmax threads] page maxima
-
   if (warp == kAttnTmaWarp) {
-    // ---- TMA producer: K and V^T pages of the item, in order
+    // ---- TMA producer: K and V^T pages of the item, in order.  The first page
+    // numbers come in one coalesced read; the rest are read a page ahead.
+    for (int i = lane; i < min(np, kAttnPtAhead); i += 32) pt_s[i] = pt[p_begin + i];
+    __syncwarp();
     if (elect_one()) {
       const int safe_pages = a.blk_slot ? a.lim[tok0] / 64 : 0;   // wholly committed pages
       const uint64_t pol = l2_policy_evict_first();
       int issued = 0;
       RingPos r;
       const uint32_t full0 = smem_u32(full), empty0 = smem_u32(empty), ring0 = smem_u32(ring);
+      int ahead = np > kAttnPtAhead ? pt[p_begin + kAttnPtAhead] : 0;
       auto issue = [&](int i) {   // page i into the ring's next stage
-        int phys = pt[p_begin + i];
+        int phys = i < kAttnPtAhead ? pt_s[i] : ahead;
+        if (i >= kAttnPtAhead && i + 1 < np) ahead = pt[p_begin + i + 1];
         if (phys < 0) {  // unmapped page: the TMA box lands out of bounds and reads zeros
           atomicExch(a.err, kErrBounds);
           phys = 0x3FFFFFFF / a.rows_per_page;
@@ -502,29 +539,38 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
       umma_commit(smem_u32(mma_done));   // retires once every MMA above has
     }
   } else {
-    // ---- softmax warps: DUP copies of each row across the 128 MMA rows
-    const int dup = R <= 32 ? 4 : (R <= 64 ? 2 : 1);
-    const int rpc = kAttnMaxRows / dup;
-    // Q rows -> swizzled smem: MMA row i holds block row i % rpc (zero past R)
+    // ---- softmax warps: Q rows -> swizzled smem (MMA row i holds block row
+    // attn_block_row(i), zero past R; rows past the last set are not read)
+    const int rows_w = warp < nbusy ? (R - warp + 3) / 4 : 0;   // rows in this warp's quarter
+    const int lanes_used = ((R + 3) / 4 + 7) / 8 * 8;
     pdl_wait();
     pdl_trigger();
-    for (int idx = threadIdx.x; idx < rows_alloc * 8; idx += kAttnSoftThreads) {
-      const int i = idx >> 3, ch = idx & 7, rr = i % rpc;
-      uint4 v = make_uint4(0, 0, 0, 0);
+    const int ch = threadIdx.x & 7, i0 = threadIdx.x >> 3;
+    uint4 v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {   // all loads in flight together
+      const int i = i0 + 16 * k, rr = attn_block_row(i);
+      v[k] = make_uint4(0, 0, 0, 0);
       if (rr < R) {
         const int t = tok0 + rr / a.G;
         const int hq = h * a.G + rr % a.G;
-        v = *reinterpret_cast<const uint4*>(a.q + (static_cast<size_t>(t) * a.Hq + hq) * 64 + ch * 8);
+        v[k] = *reinterpret_cast<const uint4*>(a.q + (static_cast<size_t>(t) * a.Hq + hq) * 64 + ch * 8);
       }
-      *reinterpret_cast<uint4*>(sQ + sw128(i, ch)) = v;
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int i = i0 + 16 * k;
+      if ((i & 31) < lanes_used) *reinterpret_cast<uint4*>(sQ + sw128(i, ch)) = v[k];
     }
     fence_proxy_async_smem();
     __syncwarp();
     if (lane == 0) mbar_arrive(smem_u32(q_full));
-    AttnSync y{s_full, s_free, p_full, empty, sP, red};
-    if (dup == 4) ok = attn_softmax<4>(a, y, tmem, np, p_begin, R, tok0, m);
-    else if (dup == 2) ok = attn_softmax<2>(a, y, tmem, np, p_begin, R, tok0, m);
-    else ok = attn_softmax<1>(a, y, tmem, np, p_begin, R, tok0, m);
+    AttnSync y{s_full, s_free, p_full, empty, sP, m_row};
+    const int nset = (rows_w + 7) / 8;
+    if (nset == 1) ok = attn_softmax<1>(a, y, tmem, warp, np, p_begin, R, tok0);
+    else if (nset == 2) ok = attn_softmax<2>(a, y, tmem, warp, np, p_begin, R, tok0);
+    else if (nset == 3) ok = attn_softmax<3>(a, y, tmem, warp, np, p_begin, R, tok0);
+    else if (nset == 4) ok = attn_softmax<4>(a, y, tmem, warp, np, p_begin, R, tok0);
   }
 
   const bool all_ok = __syncthreads_and(ok);
@@ -536,9 +582,10 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
   }
   __syncthreads();
   // the row's O and its sum (O's column 64) from TMEM (rows < R)
-  const int r = threadIdx.x;
+  const int r = warp < kAttnSoftWarps ? attn_block_row(threadIdx.x) : kAttnMaxRows;   // block row
   const bool row_thread = r < R;
   float o[64];
+  float m = -INFINITY, l = 0.f;   // the row's running max (log2 units) and sum
   if (warp < 4) {
     tc_fence_after();
     uint32_t o0[32], o1[32];
@@ -546,6 +593,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
     tmem_ld32_nowait(tmem + (static_cast<uint32_t>(warp * 32) << 16) + 128 + 32, o1);
     const uint32_t l1 = tmem_ld1(tmem + (static_cast<uint32_t>(warp * 32) << 16) + 192);
     tmem_wait_ld();
+    m = m_row[threadIdx.x];
     l = __uint_as_float(l1);
 #pragma unroll
     for (int k = 0; k < 32; ++k) {
