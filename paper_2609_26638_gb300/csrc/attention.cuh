@@ -51,10 +51,15 @@
 
 namespace gs {
 
-constexpr int kAttnStages = 3;             // K/V page pairs in flight
+// K pages and V^T pages have rings of their own: a K page is done with S, a V^T
+// page only a softmax and a P V later.  In one ring of 3 pairs a copy went out
+// when P V of its predecessor ended and was wanted one page later (the MMA warp
+// waited 610 of 1,700 cycles per page for it, 32 x U[1024, 6144] slots); here a
+// K copy has 4 pages of lead and a V^T copy 3, in what two CTAs per SM can hold.
+constexpr int kAttnKStages = 4, kAttnVStages = 3;
 constexpr int kAttnPageBytes = 64 * 128;  // 64 x 64 fp16
 constexpr int kAttnOnesBytes = 16 * 128;  // 16 rows of fp16 ones after each V^T page
-constexpr int kAttnStageBytes = 2 * kAttnPageBytes + kAttnOnesBytes;
+constexpr int kAttnVStageBytes = kAttnPageBytes + kAttnOnesBytes;
 constexpr int kAttnRow = 68;              // partial row: O[64], m, l, 2 pad (272 B)
 constexpr int kAttnMaxRows = 128;         // rows of one query block (the MMA's M)
 constexpr int kAttnMaxCluster = 16;       // items merged inside a cluster (16: non-portable size)
@@ -65,10 +70,11 @@ constexpr int kAttnTmaWarp = kAttnSoftWarps, kAttnMmaWarp = kAttnSoftWarps + 1;
 constexpr int kAttnTmemCols = 256;        // S[2] at columns 0, 64; O at 128
 constexpr int kAttnPtAhead = 64;         // page numbers an item reads up front
 constexpr float kAttnRescale = 8.0f;      // log2 growth of the max that forces a rescale
-constexpr int kAttnRingBytes = kAttnStages * kAttnStageBytes;
-// Q [128][128 B] | P[2] [128][128 B] | ring | barriers.  After the pages are
-// done, Q and P hold the owner-grouped rows (cluster) and the ring the
-// received rows or the merge's (m, l) tables.
+constexpr int kAttnKRingBytes = kAttnKStages * kAttnPageBytes;
+constexpr int kAttnRingBytes = kAttnKRingBytes + kAttnVStages * kAttnVStageBytes;
+// Q [128][128 B] | P[2] [128][128 B] | K ring | V^T ring | barriers.  After the
+// pages are done, Q and P hold the owner-grouped rows (cluster) and the rings
+// the received rows or the merge's (m, l) tables.
 constexpr int kAttnQOff = 0;
 constexpr int kAttnPOff = kAttnMaxRows * 128;
 constexpr int kAttnRingOff = kAttnPOff + 2 * kAttnMaxRows * 128;
@@ -77,6 +83,11 @@ constexpr int kAttnSmemBytes = 1024 + kAttnBarOff + 256 + kAttnMaxRows * 4 + kAt
 constexpr int kAttnRowsFloats = (kAttnMaxRows + kAttnMaxCluster) * kAttnRow;
 static_assert(kAttnRingOff >= kAttnRowsFloats * 4 && kAttnRingBytes >= kAttnRowsFloats * 4,
               "Q + P hold the owner-grouped rows, the ring the received rows");
+static_assert(kAttnRingOff >= 2 * kAttnMaxCluster * kAttnMaxRows * 4, "Q + P hold a cluster's tables");
+// Items one global merge takes (an interface limit: the tables of m and l, 1 KB
+// per item, have to fit the ring).
+constexpr int kAttnMaxMergeItems = 54;
+static_assert(kAttnMaxMergeItems * 2 * kAttnMaxRows * 4 <= kAttnRingBytes, "merge tables");
 
 struct AttnArgs {
   const __half* q;            // [T, Hq, 64]
@@ -91,6 +102,7 @@ struct AttnArgs {
   int QB;                     // tokens per sequence window (prefill: per block)
   int QS, n_sub;              // tokens per query block; blocks per window
   int Hq, Hkv, G;
+  int g_magic;                // ceil(2^16 / G): r / G = r * g_magic >> 16 for block rows r < 128
   long long kv_row_base;      // first KV-map row of this layer
   int rows_per_page;          // 2 * Hkv * 64
   int split_pages;            // SP: pages per item
@@ -102,10 +114,6 @@ struct AttnArgs {
 };
 
 __host__ __device__ inline int attn_max_smem_bytes() { return kAttnSmemBytes; }
-// The merge keeps m and l of every (item, row) in the idle ring.
-__host__ __device__ inline int attn_max_merge_items(int /*rows*/) {
-  return kAttnRingBytes / 4 / (2 * kAttnMaxRows);
-}
 
 __device__ __forceinline__ uint32_t sw128(int row, int chunk) {
   return static_cast<uint32_t>(row * 128 + ((chunk ^ (row & 7)) << 4));
@@ -126,18 +134,6 @@ __device__ __forceinline__ void tmem_ld_16x256b_x8(uint32_t taddr, uint32_t (&r)
         "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
         "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_st_16x256b_x8(uint32_t taddr, const uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.16x256b.x8.b32 [%0], "
-      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(taddr),
-      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-      "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]),
-      "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]),
-      "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]),
-      "r"(r[29]), "r"(r[30]), "r"(r[31])
-      : "memory");
 }
 __device__ __forceinline__ void tmem_ld_16x256b_x1(uint32_t taddr, uint32_t (&r)[4]) {
   asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0, %1, %2, %3}, [%4];"
@@ -174,42 +170,46 @@ __device__ __forceinline__ float fmax3(float x, float y, float z) {
 // Barriers and buffers the softmax warps share with the MMA warp.
 struct AttnSync {
   uint64_t *s_full, *s_free, *p_full;
-  uint64_t* empty;   // [stages] O += P V of the stage's page retired
-  uint8_t* sP;       // [2][128][128 B]
+  uint64_t* v_empty;   // [V stages] O += P V of the stage's page retired
+  uint8_t* sP;         // [2][128][128 B]
   float* m_row;      // [128] per MMA row: the final running max
 };
 
 // MMA row (TMEM lane) -> block row, and back.
 __device__ __forceinline__ int attn_block_row(int mrow) { return (mrow & 31) * 4 + (mrow >> 5); }
 
-// Online softmax over the item's pages, for a warp whose lane quarter holds at
-// most 8 NSET rows.  S comes from TMEM in the 16x256b layout, so a row is
-// spread over four neighbouring threads and set q (rows 8 q .. 8 q + 7 of the
-// quarter) costs a thread 16 columns, whatever the number of rows in the block
-// is: 34 rows (a 17-token window, GQA 2) cost 16 or 32 exponentials per thread
-// and page.  Per page: S, mask and scale, the row's maximum (two shuffles);
-// the row's running max m (log2 units) only moves when a page raises it by
-// more than 2^8 (always on the first page, rarely after).  A rise rescales O
-// and the row sum in O's column 64 (the previous O += P V must have retired);
-// then P_j = exp2(s - m) as fp16 into the P tile.  No step of a page needs
-// another warp: the warps meet only on the MMA warp's barriers.  Bound by the
-// serial chain of a page (TMEM load, max, exponentials, P store, fence).
+// Online softmax over the item's pages for one warp and the rows of its lane
+// quarter.  S comes from TMEM in the 16x256b layout, so a row is spread over
+// four neighbouring threads and a set of 8 rows costs a thread 16 columns,
+// whatever the number of rows in the block is: 34 rows (a 17-token window,
+// GQA 2) cost 16 or 32 exponentials per thread and page.  Per page: S, mask and
+// scale, the row's maximum (two shuffles); the row's running max m (log2 units)
+// only moves when a page raises it by more than 2^8 (always on the first page,
+// rarely after).  A rise rescales O and the row sum in O's column 64 (the
+// previous O += P V must have retired); then P_j = exp2(s - m) as fp16 into the
+// P tile.  No step of a page needs another warp: the warps meet only on the MMA
+// warp's barriers.  Bound by the serial chain of a page (TMEM load, max,
+// exponentials, P store, fence).
+//
+// The quarter's two 16-lane halves run through one rolled loop and the mask and
+// the rescale are loops too: every CTA of a launch fetches this code again (the
+// SM's instruction cache does not hold a kernel of 100 KB), and the four
+// unrolled variants this replaces spent 10 k of a CTA's 34 k cycles on that.
 // Waits are bounded; a warp whose wait ran out keeps arriving on the MMA
 // warp's barriers to the last page.  Returns false if a wait ran out.
-template <int NSET>
 __device__ __forceinline__ bool attn_softmax(const AttnArgs& a, const AttnSync& y, uint32_t tmem,
-                                             int warp, int np, int p_begin, int R, int tok0) {
-  constexpr int NH = (NSET + 1) / 2;   // 16-lane halves of the quarter
+                                             int warp, int rows_w, int np, int p_begin, int R,
+                                             int tok0) {
   const int lane = threadIdx.x & 31;
   const int quad = lane & 3;
-  float m[NSET];
-  int lim[NSET];
+  const int nset = (rows_w + 7) / 8;   // sets of 8 rows, two per half
+  float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+  int lim[4];
   int full_lim = 0x7FFFFFFF;   // every row of the warp sees the keys up to here
 #pragma unroll
-  for (int q = 0; q < NSET; ++q) {
+  for (int q = 0; q < 4; ++q) {
     const int rr = (8 * q + (lane >> 2)) * 4 + warp;
-    m[q] = -INFINITY;
-    lim[q] = rr < R ? a.lim[tok0 + rr / a.G] : -1;
+    lim[q] = rr < R ? a.lim[tok0 + (rr * a.g_magic >> 16)] : -1;
     if (rr < R) full_lim = min(full_lim, lim[q]);
   }
   full_lim = __reduce_min_sync(0xFFFFFFFFu, full_lim);
@@ -224,113 +224,117 @@ __device__ __forceinline__ bool attn_softmax(const AttnArgs& a, const AttnSync& 
     if (ok) ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, a.err)) != 0;
     return ok;
   };
+  RingPos prev;   // V^T ring position of page j - 1
+  bool pv_seen = true;   // O += P V of page j - 1 is known to have retired
+#pragma unroll 1
   for (int j = 0; j < np; ++j) {
     const int buf = j & 1;
     const bool have = wwait(s_full0 + 8 * buf, (j >> 1) & 1);
-    // 1. S_j; the buffer is free once every warp has read it
-    uint32_t sr[NH][32];
+    const int key0 = (p_begin + j) * 64;
     if (have) {
       tc_fence_after();
-#pragma unroll
-      for (int hf = 0; hf < NH; ++hf)
-        tmem_ld_16x256b_x8(trow + (static_cast<uint32_t>(16 * hf) << 16) + buf * 64, sr[hf]);
-      tmem_wait_ld();
-    }
-    tc_fence_before();
-    __syncwarp();
-    if (lane == 0) mbar_arrive(s_free0 + 8 * buf);
-    if (have) {
-      // 2. mask: keys past the row's limit (only on a window's last pages)
-      const int key0 = (p_begin + j) * 64;
-      if (key0 + 63 > full_lim) {
-#pragma unroll
-        for (int q = 0; q < NSET; ++q)
+#pragma unroll 1
+      for (int hf = 0; 2 * hf < nset; ++hf) {
+        const bool two = 2 * hf + 1 < nset;   // the half's second set holds rows
+        float mh[2] = {hf ? m[2] : m[0], hf ? m[3] : m[1]};
+        const uint32_t half = static_cast<uint32_t>(16 * hf) << 16;
+        // 1. S_j of the half; the buffer is free once every warp has read it
+        uint32_t sr[32];
+        tmem_ld_16x256b_x8(trow + half + buf * 64, sr);
+        tmem_wait_ld();
+        if (2 * hf + 2 >= nset) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(s_free0 + 8 * buf);
+        }
+        // 2. mask: keys past the row's limit (only on a window's last pages)
+        if (key0 + 63 > full_lim) {
+          const int l0 = hf ? lim[2] : lim[0], l1 = hf ? lim[3] : lim[1];
 #pragma unroll
           for (int k = 0; k < 16; ++k) {
             const int key = key0 + 8 * (k >> 1) + 2 * quad + (k & 1);
-            uint32_t& v = sr[q >> 1][4 * (k >> 1) + 2 * (q & 1) + (k & 1)];
-            v = key <= lim[q] ? v : 0xFF800000u;
+            uint32_t& v0 = sr[4 * (k >> 1) + (k & 1)];
+            uint32_t& v1 = sr[4 * (k >> 1) + 2 + (k & 1)];
+            v0 = key <= l0 ? v0 : 0xFF800000u;
+            v1 = key <= l1 ? v1 : 0xFF800000u;
           }
-      }
-      // 3. the row's page max (of the unscaled scores; the scale is positive)
-      //    over the four threads of the row; does any row rise by more than 2^8?
-      float pm[NSET];
-      bool rise[NSET], any = false;
+        }
+        // 3. the rows' page max (of the unscaled scores; the scale is positive)
+        //    over the four threads of a row; does any row rise by more than 2^8?
+        float pm[2];
 #pragma unroll
-      for (int q = 0; q < NSET; ++q) {
-        auto S = [&](int k) {
-          return __uint_as_float(sr[q >> 1][4 * (k >> 1) + 2 * (q & 1) + (k & 1)]);
-        };
-        float t = fmax3(fmax3(S(0), S(1), S(2)), fmax3(S(3), S(4), S(5)), fmax3(S(6), S(7), S(8)));
-        t = fmax3(t, fmax3(S(9), S(10), S(11)), fmax3(S(12), S(13), fmaxf(S(14), S(15))));
-        t = fmaxf(t, __shfl_xor_sync(0xFFFFFFFFu, t, 1));
-        t = fmaxf(t, __shfl_xor_sync(0xFFFFFFFFu, t, 2));
-        pm[q] = t * kScaleLog2;
-        rise[q] = pm[q] > m[q] + kAttnRescale;
-        any |= rise[q];
-      }
-      // 4. a rise rescales O and the row sum first.  tcgen05.ld / st are
-      //    warp-collective: a warp with any rising row rescales all its rows,
-      //    the others by exactly 1.
-      if (__any_sync(0xFFFFFFFFu, any)) {
-        float alpha[2 * NH];
+        for (int q = 0; q < 2; ++q) {
+          auto S = [&](int k) { return __uint_as_float(sr[4 * (k >> 1) + 2 * q + (k & 1)]); };
+          float t = fmax3(fmax3(S(0), S(1), S(2)), fmax3(S(3), S(4), S(5)), fmax3(S(6), S(7), S(8)));
+          t = fmax3(t, fmax3(S(9), S(10), S(11)), fmax3(S(12), S(13), fmaxf(S(14), S(15))));
+          t = fmaxf(t, __shfl_xor_sync(0xFFFFFFFFu, t, 1));
+          t = fmaxf(t, __shfl_xor_sync(0xFFFFFFFFu, t, 2));
+          pm[q] = t * kScaleLog2;
+        }
+        const bool rise0 = pm[0] > mh[0] + kAttnRescale;
+        const bool rise1 = two && pm[1] > mh[1] + kAttnRescale;
+        // 4. a rise rescales O and the row sum first.  tcgen05.ld / st are
+        //    warp-collective: a half with any rising row rescales all its rows,
+        //    the others by exactly 1.
+        if (__any_sync(0xFFFFFFFFu, rise0 || rise1)) {
+          const float al0 = !rise0 ? 1.f : (mh[0] == -INFINITY ? 0.f : exp2f(mh[0] - pm[0]));
+          const float al1 = !rise1 ? 1.f : (mh[1] == -INFINITY ? 0.f : exp2f(mh[1] - pm[1]));
+          if (rise0) mh[0] = pm[0];
+          if (rise1) mh[1] = pm[1];
+          if (hf) {
+            m[2] = mh[0];
+            m[3] = mh[1];
+          } else {
+            m[0] = mh[0];
+            m[1] = mh[1];
+          }
+          if (!pv_seen) pv_seen = wwait(smem_u32(&y.v_empty[prev.s]), prev.ph);
+          if (j > 0 && pv_seen) {
+            tc_fence_after();
+            const uint32_t o = trow + half + 128;
+#pragma unroll 1
+            for (int cg = 0; cg < 9; ++cg) {   // 8 columns each; the last: the row sums
+              uint32_t v[4];
+              tmem_ld_16x256b_x1(o + 8 * cg, v);
+              tmem_wait_ld();
 #pragma unroll
-        for (int q = 0; q < 2 * NH; ++q) {
-          alpha[q] = 1.f;
-          if (q < NSET) {
-            const int qq = q < NSET ? q : 0;
-            if (rise[qq]) {
-              alpha[q] = m[qq] == -INFINITY ? 0.f : exp2f(m[qq] - pm[qq]);
-              m[qq] = pm[qq];
+              for (int k = 0; k < 4; ++k)
+                v[k] = __float_as_uint((k < 2 ? al0 : al1) * __uint_as_float(v[k]));
+              tmem_st_16x256b_x1(o + 8 * cg, v);
             }
+            tmem_wait_st();
           }
         }
-        if (j > 0 && wwait(smem_u32(&y.empty[(j - 1) % kAttnStages]), ((j - 1) / kAttnStages) & 1)) {
-          tc_fence_after();
+        // 5. P_j = exp2(s - m) (fp16) into the rows of the P tile
+        const uint32_t prow = p0 + buf * (kAttnMaxRows * 128) + hf * (16 * 128);
+        auto put = [&](int q, float mq, uint32_t row) {
+          const float sub = (mq == -INFINITY) ? 0.f : mq;
 #pragma unroll
-          for (int hf = 0; hf < NH; ++hf) {
-            const uint32_t o = trow + (static_cast<uint32_t>(16 * hf) << 16) + 128;
-            uint32_t v[32], l4[4];
-            tmem_ld_16x256b_x8(o, v);
-            tmem_ld_16x256b_x1(o + 64, l4);   // the row sums, O's columns 64..71
-            tmem_wait_ld();
-#pragma unroll
-            for (int k = 0; k < 32; ++k)
-              v[k] = __float_as_uint(alpha[2 * hf + ((k >> 1) & 1)] * __uint_as_float(v[k]));
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-              l4[k] = __float_as_uint(alpha[2 * hf + (k >> 1)] * __uint_as_float(l4[k]));
-            tmem_st_16x256b_x8(o, v);
-            tmem_st_16x256b_x1(o + 64, l4);
+          for (int jj = 0; jj < 8; ++jj) {
+            const float x0 = ex2_sfu(fmaf(__uint_as_float(sr[4 * jj + 2 * q]), kScaleLog2, -sub));
+            const float x1 = ex2_sfu(fmaf(__uint_as_float(sr[4 * jj + 2 * q + 1]), kScaleLog2, -sub));
+            const __half2 hv = __floats2half2_rn(x0, x1);
+            asm volatile("st.shared.b32 [%0], %1;" ::"r"(row ^ (jj << 4)),
+                         "r"(*reinterpret_cast<const uint32_t*>(&hv))
+                         : "memory");
           }
-          tmem_wait_st();
-        }
-      }
-      // 5. P_j = exp2(s - m) (fp16) into the rows of the P tile
-#pragma unroll
-      for (int q = 0; q < NSET; ++q) {
-        const float sub = (m[q] == -INFINITY) ? 0.f : m[q];
-        const uint32_t prow = p0 + buf * (kAttnMaxRows * 128) + q * (8 * 128);
-#pragma unroll
-        for (int jj = 0; jj < 8; ++jj) {
-          const int k = 4 * jj + 2 * (q & 1);
-          const float x0 = ex2_sfu(fmaf(__uint_as_float(sr[q >> 1][k]), kScaleLog2, -sub));
-          const float x1 = ex2_sfu(fmaf(__uint_as_float(sr[q >> 1][k + 1]), kScaleLog2, -sub));
-          const __half2 hv = __floats2half2_rn(x0, x1);
-          asm volatile("st.shared.b32 [%0], %1;" ::"r"(prow ^ (jj << 4)),
-                       "r"(*reinterpret_cast<const uint32_t*>(&hv))
-                       : "memory");
-        }
+        };
+        put(0, mh[0], prow);
+        if (two) put(1, mh[1], prow + 8 * 128);
       }
       fence_proxy_async_smem();
+    } else if (lane == 0) {
+      mbar_arrive(s_free0 + 8 * buf);
     }
     tc_fence_before();
     __syncwarp();
     if (lane == 0) mbar_arrive(p_full0 + 8 * buf);
+    if (j > 0) prev.next(kAttnVStages);
+    pv_seen = false;
   }
   if (quad == 0) {
 #pragma unroll
-    for (int q = 0; q < NSET; ++q) y.m_row[warp * 32 + 8 * q + (lane >> 2)] = m[q];
+    for (int q = 0; q < 4; ++q) y.m_row[warp * 32 + 8 * q + (lane >> 2)] = m[q];
   }
   return ok;
 }
@@ -345,20 +349,23 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
   constexpr int rows_alloc = kAttnMaxRows;
   uint8_t* sQ = smem + kAttnQOff;
   uint8_t* sP = smem + kAttnPOff;                        // [2][128][128 B]
-  uint8_t* ring = smem + kAttnRingOff;                   // [stage][K | V^T]
+  uint8_t* ring = smem + kAttnRingOff;                   // K pages
+  uint8_t* vring = ring + kAttnKRingBytes;               // V^T pages, 16 rows of ones behind each
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kAttnBarOff);
-  uint64_t* full = bars;                                 // [stages] TMA landed
-  uint64_t* empty = bars + kAttnStages;                  // [stages] PV of the page done
-  uint64_t* s_full = bars + 2 * kAttnStages;             // [2] S in TMEM
-  uint64_t* s_free = s_full + 2;                         // [2] S read by the 4 softmax warps
-  uint64_t* p_full = s_full + 4;                         // [2] P in smem (4 warp arrivals)
-  uint64_t* mma_done = s_full + 7;                       // every MMA of this CTA retired
-  uint64_t* recv_bar = s_full + 8;
-  uint64_t* q_full = s_full + 9;                         // Q tile in smem (4 warp arrivals)
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_full + 12);
-  // [0] max limit, [1] last-item flag, [2] pages the MMA warp took, [3] pages
-  // issued, [4] sequence active, [5] page-table row
-  int* s_int = reinterpret_cast<int*>(s_full + 13);
+  uint64_t* k_full = bars;                               // [K stages] TMA landed
+  uint64_t* k_empty = k_full + kAttnKStages;             // [K stages] S of the page done
+  uint64_t* v_full = k_empty + kAttnKStages;             // [V stages] TMA landed
+  uint64_t* v_empty = v_full + kAttnVStages;             // [V stages] PV of the page done
+  uint64_t* s_full = v_empty + kAttnVStages;             // [2] S in TMEM
+  uint64_t* s_free = s_full + 2;                         // [2] S read by the softmax warps
+  uint64_t* p_full = s_full + 4;                         // [2] P in smem (softmax warps' arrivals)
+  uint64_t* mma_done = s_full + 6;                       // every MMA of this CTA retired
+  uint64_t* recv_bar = s_full + 7;
+  uint64_t* q_full = s_full + 8;                         // Q tile in smem (4 warp arrivals)
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_full + 9);
+  // [0] max limit, [1] last-item flag, [2] K and [3] V^T pages the MMA warp
+  // took, [4] K and [5] V^T pages issued, [6] sequence active, [7] page-table row
+  int* s_int = reinterpret_cast<int*>(s_full + 10);
   float* m_row = reinterpret_cast<float*>(s_int + 8);    // [128] running max per MMA row
   int* pt_s = reinterpret_cast<int*>(m_row + kAttnMaxRows);   // the item's first page numbers
 
@@ -386,15 +393,12 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
     const int mxl = __reduce_max_sync(0xFFFFFFFFu, max(max(lm[0], lm[1]), max(lm[2], lm[3])));
     if (lane == 0) {
       s_int[0] = mxl;
-      s_int[4] = act;
-      s_int[5] = sl;
+      s_int[6] = act;
+      s_int[7] = sl;
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      for (int s = 0; s < kAttnStages; ++s) {
-        mbar_init(smem_u32(&full[s]), 1);
-        mbar_init(smem_u32(&empty[s]), 1);
-      }
+      for (int s = 0; s < 2 * (kAttnKStages + kAttnVStages); ++s) mbar_init(smem_u32(&bars[s]), 1);
       for (int i = 0; i < 2; ++i) {
         mbar_init(smem_u32(&s_full[i]), 1);
         mbar_init(smem_u32(&s_free[i]), nbusy);   // one arrival per softmax warp with rows
@@ -403,15 +407,14 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
       mbar_init(smem_u32(mma_done), 1);
       mbar_init(smem_u32(q_full), kAttnSoftWarps);
       mbar_init(smem_u32(recv_bar), 1);
-      s_int[2] = 0;
-      s_int[3] = 0;
+      s_int[2] = s_int[3] = s_int[4] = s_int[5] = 0;
       fence_mbar_init();
     }
   } else if (warp < kAttnSoftWarps) {
     // the ones rows after every V^T page: O += P [V | 1] puts the row sum in O's column 64
-    for (int i = threadIdx.x - 64; i < kAttnStages * kAttnOnesBytes / 16; i += 64) {
+    for (int i = threadIdx.x - 64; i < kAttnVStages * kAttnOnesBytes / 16; i += 64) {
       const int st = i / (kAttnOnesBytes / 16), off = i % (kAttnOnesBytes / 16);
-      *reinterpret_cast<uint4*>(ring + st * kAttnStageBytes + 2 * kAttnPageBytes + off * 16) =
+      *reinterpret_cast<uint4*>(vring + st * kAttnVStageBytes + kAttnPageBytes + off * 16) =
           make_uint4(0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u);
     }
     fence_proxy_async_smem();
@@ -424,11 +427,11 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const int maxlim = s_int[0], slot = s_int[5];
+  const int maxlim = s_int[0], slot = s_int[7];
   const int npages_blk = maxlim / 64 + 1;
   const int SP = a.split_pages;
   const int nitems = (npages_blk + SP - 1) / SP;
-  const bool active = s_int[4] != 0;
+  const bool active = s_int[6] != 0;
   const bool bad = maxlim < 0 || npages_blk > a.pt_stride || slot < 0 || nitems > a.max_items ||
                    R > kAttnMaxRows;
   const bool in_cluster = a.cluster && nitems > 1;
@@ -458,35 +461,63 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
     if (elect_one()) {
       const int safe_pages = a.blk_slot ? a.lim[tok0] / 64 : 0;   // wholly committed pages
       const uint64_t pol = l2_policy_evict_first();
-      int issued = 0;
-      RingPos r;
-      const uint32_t full0 = smem_u32(full), empty0 = smem_u32(empty), ring0 = smem_u32(ring);
+      RingPos rk, rv;
+      const uint32_t k_full0 = smem_u32(k_full), k_empty0 = smem_u32(k_empty);
+      const uint32_t v_full0 = smem_u32(v_full), v_empty0 = smem_u32(v_empty);
+      const uint32_t k0 = smem_u32(ring), v0 = smem_u32(vring);
       int ahead = np > kAttnPtAhead ? pt[p_begin + kAttnPtAhead] : 0;
-      auto issue = [&](int i) {   // page i into the ring's next stage
+      int vrow = 0;   // pool row of the page whose V^T copy is next
+      auto issue_k = [&](int i) {   // returns the page's V^T row
         int phys = i < kAttnPtAhead ? pt_s[i] : ahead;
         if (i >= kAttnPtAhead && i + 1 < np) ahead = pt[p_begin + i + 1];
         if (phys < 0) {  // unmapped page: the TMA box lands out of bounds and reads zeros
           atomicExch(a.err, kErrBounds);
           phys = 0x3FFFFFFF / a.rows_per_page;
         }
-        const long long row = a.kv_row_base + static_cast<long long>(phys) * a.rows_per_page;
-        const uint32_t fb = full0 + 8 * r.s, st = ring0 + r.s * kAttnStageBytes;
-        mbar_arrive_expect_tx(fb, 2 * kAttnPageBytes);   // K and V^T (the ones rows stay)
-        tma_load_2d(st, &tmKV, 0, static_cast<int>(row + h * 64), fb, pol);
-        tma_load_2d(st + kAttnPageBytes, &tmKV, 0, static_cast<int>(row + (a.Hkv + h) * 64), fb, pol);
-        r.next(kAttnStages);
+        const int row = static_cast<int>(a.kv_row_base + static_cast<long long>(phys) * a.rows_per_page);
+        const uint32_t fb = k_full0 + 8 * rk.s;
+        mbar_arrive_expect_tx(fb, kAttnPageBytes);
+        tma_load_2d(k0 + rk.s * kAttnPageBytes, &tmKV, 0, row + h * 64, fb, pol);
+        rk.next(kAttnKStages);
+        s_int[4] = i + 1;
+        return row + (a.Hkv + h) * 64;
       };
-      while (issued < min(np, kAttnStages) && p_begin + issued < safe_pages) issue(issued++);
+      auto issue_v = [&](int i, int row) {
+        const uint32_t fb = v_full0 + 8 * rv.s;
+        mbar_arrive_expect_tx(fb, kAttnPageBytes);   // the ones rows stay
+        tma_load_2d(v0 + rv.s * kAttnVStageBytes, &tmKV, 0, row, fb, pol);
+        rv.next(kAttnVStages);
+        s_int[5] = i + 1;
+      };
+      // K of page i, then V^T of page i - 1: S runs a page ahead of P V
+      int i = 0;
+      const int npre = min(np, min(safe_pages - p_begin, kAttnVStages));
+#pragma unroll 1
+      for (; i < npre; ++i) {
+        if (i > 0) issue_v(i - 1, vrow);
+        vrow = issue_k(i);
+      }
       pdl_wait();
       pdl_trigger();
-      while (issued < np && ok) {
-        if (issued >= kAttnStages && !mbar_wait(empty0 + 8 * r.s, r.ph ^ 1, a.err)) {
-          ok = false;
-          break;
+#pragma unroll 1
+      for (; i <= np && ok; ++i) {
+        int next_vrow = 0;
+        if (i < np) {
+          if (i >= kAttnKStages && !mbar_wait(k_empty0 + 8 * rk.s, rk.ph ^ 1, a.err)) {
+            ok = false;
+            break;
+          }
+          next_vrow = issue_k(i);
         }
-        issue(issued++);
+        if (i > 0) {
+          if (i > kAttnVStages && !mbar_wait(v_empty0 + 8 * rv.s, rv.ph ^ 1, a.err)) {
+            ok = false;
+            break;
+          }
+          issue_v(i - 1, vrow);
+        }
+        vrow = next_vrow;
       }
-      s_int[3] = issued;
     } else {
       pdl_wait();
       pdl_trigger();
@@ -501,40 +532,49 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
       const uint64_t qdesc = umma_desc_sw128(smem_u32(sQ));
       const uint64_t pdesc0 = umma_desc_sw128(smem_u32(sP));
       const uint64_t kdesc0 = umma_desc_sw128(smem_u32(ring));
-      const uint32_t full0 = smem_u32(full), empty0 = smem_u32(empty);
+      const uint64_t vdesc0 = umma_desc_sw128(smem_u32(vring));
+      const uint32_t k_full0 = smem_u32(k_full), k_empty0 = smem_u32(k_empty);
+      const uint32_t v_full0 = smem_u32(v_full), v_empty0 = smem_u32(v_empty);
       const uint32_t s_full0 = smem_u32(s_full), s_free0 = smem_u32(s_free), p_full0 = smem_u32(p_full);
-      RingPos rs, rv;   // ring stages of the next S and the next PV
+      RingPos rk, rv;   // ring stages of the next S and the next PV
       auto issue_s = [&](int j) -> bool {
         const int buf = j & 1;
-        if (!mbar_wait(full0 + 8 * rs.s, rs.ph, a.err)) return false;
+        if (!mbar_wait(k_full0 + 8 * rk.s, rk.ph, a.err)) return false;
         s_int[2] = j + 1;
         if (j >= 2 && !mbar_wait(s_free0 + 8 * buf, ((j >> 1) + 1) & 1, a.err)) return false;
         tc_fence_after();
-        const uint64_t kdesc = kdesc0 + rs.s * (kAttnStageBytes >> 4);
+        const uint64_t kdesc = kdesc0 + rk.s * (kAttnPageBytes >> 4);
 #pragma unroll
         for (int k = 0; k < 4; ++k)
           umma_f16(tmem + buf * 64, qdesc + 2 * k, kdesc + 2 * k, idesc, k > 0 ? 1u : 0u);
         umma_commit(s_full0 + 8 * buf);
-        rs.next(kAttnStages);
+        umma_commit(k_empty0 + 8 * rk.s);
+        rk.next(kAttnKStages);
         return true;
       };
       if (!mbar_wait(smem_u32(q_full), 0, a.err)) ok = false;   // Q tile written
       if (ok) ok = issue_s(0);
+#pragma unroll 1
       for (int j = 0; j < np && ok; ++j) {
         if (j + 1 < np && !(ok = issue_s(j + 1))) break;
         const int buf = j & 1;
+        if (!mbar_wait(v_full0 + 8 * rv.s, rv.ph, a.err)) {
+          ok = false;
+          break;
+        }
+        s_int[3] = j + 1;
         if (!mbar_wait(p_full0 + 8 * buf, (j >> 1) & 1, a.err)) {
           ok = false;
           break;
         }
         tc_fence_after();
         const uint64_t pdesc = pdesc0 + buf * (kAttnMaxRows * 128 >> 4);
-        const uint64_t vdesc = kdesc0 + ((rv.s * kAttnStageBytes + kAttnPageBytes) >> 4);
+        const uint64_t vdesc = vdesc0 + rv.s * (kAttnVStageBytes >> 4);
 #pragma unroll
         for (int k = 0; k < 4; ++k)
           umma_f16(tmem + 128, pdesc + 2 * k, vdesc + 2 * k, idesc_pv, (j > 0 || k > 0) ? 1u : 0u);
-        umma_commit(empty0 + 8 * rv.s);
-        rv.next(kAttnStages);
+        umma_commit(v_empty0 + 8 * rv.s);
+        rv.next(kAttnVStages);
       }
       umma_commit(smem_u32(mma_done));   // retires once every MMA above has
     }
@@ -552,8 +592,9 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
       const int i = i0 + 16 * k, rr = attn_block_row(i);
       v[k] = make_uint4(0, 0, 0, 0);
       if (rr < R) {
-        const int t = tok0 + rr / a.G;
-        const int hq = h * a.G + rr % a.G;
+        const int tt = rr * a.g_magic >> 16;
+        const int t = tok0 + tt;
+        const int hq = h * a.G + rr - tt * a.G;
         v[k] = *reinterpret_cast<const uint4*>(a.q + (static_cast<size_t>(t) * a.Hq + hq) * 64 + ch * 8);
       }
     }
@@ -565,22 +606,28 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
     fence_proxy_async_smem();
     __syncwarp();
     if (lane == 0) mbar_arrive(smem_u32(q_full));
-    AttnSync y{s_full, s_free, p_full, empty, sP, m_row};
-    const int nset = (rows_w + 7) / 8;
-    if (nset == 1) ok = attn_softmax<1>(a, y, tmem, warp, np, p_begin, R, tok0);
-    else if (nset == 2) ok = attn_softmax<2>(a, y, tmem, warp, np, p_begin, R, tok0);
-    else if (nset == 3) ok = attn_softmax<3>(a, y, tmem, warp, np, p_begin, R, tok0);
-    else if (nset == 4) ok = attn_softmax<4>(a, y, tmem, warp, np, p_begin, R, tok0);
+    AttnSync y{s_full, s_free, p_full, v_empty, sP, m_row};
+    if (rows_w > 0) ok = attn_softmax(a, y, tmem, warp, rows_w, np, p_begin, R, tok0);
   }
 
-  const bool all_ok = __syncthreads_and(ok);
   // every MMA retired and every TMA copy landed before TMEM and the ring are reused
-  if (warp == kAttnMmaWarp && lane == 0) mbar_wait(smem_u32(mma_done), 0, a.err);
-  if (warp == kAttnTmaWarp && lane == 0) {
-    for (int i = s_int[2]; i < s_int[3]; ++i)
-      mbar_wait(smem_u32(&full[i % kAttnStages]), (i / kAttnStages) & 1, a.err);
+  if (warp == kAttnTmaWarp) {
+    __syncwarp();   // the elected thread's page counts are written
+  } else {
+    mbar_wait(smem_u32(mma_done), 0, a.err);
   }
-  __syncthreads();
+  const bool all_ok = __syncthreads_and(ok);
+  if (!all_ok) {   // a wait ran out: pages that were issued and not taken may still be landing
+    if (threadIdx.x == 0) {
+#pragma unroll 1
+      for (int i = s_int[2]; i < s_int[4]; ++i)
+        mbar_wait(smem_u32(&k_full[i % kAttnKStages]), (i / kAttnKStages) & 1, a.err);
+#pragma unroll 1
+      for (int i = s_int[3]; i < s_int[5]; ++i)
+        mbar_wait(smem_u32(&v_full[i % kAttnVStages]), (i / kAttnVStages) & 1, a.err);
+    }
+    __syncthreads();
+  }
   // the row's O and its sum (O's column 64) from TMEM (rows < R)
   const int r = warp < kAttnSoftWarps ? attn_block_row(threadIdx.x) : kAttnMaxRows;   // block row
   const bool row_thread = r < R;
@@ -602,17 +649,20 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
     }
   }
   tc_fence_before();
-  __syncthreads();
-  if (warp == kAttnMmaWarp) {
-    tc_fence_after();
-    tmem_dealloc(tmem, kAttnTmemCols);
-  }
 
+  // (the MMA warp frees TMEM behind the barrier that follows the row stores)
+  auto free_tmem = [&] {
+    if (warp == kAttnMmaWarp) {
+      tc_fence_after();
+      tmem_dealloc(tmem, kAttnTmemCols);
+    }
+  };
   if (nitems == 1) {   // the block's only item: its rows are final
     if (row_thread && all_ok) {
       const float inv = 1.0f / l;
-      const int t = tok0 + r / a.G;
-      const int hq = h * a.G + r % a.G;
+      const int tt = r * a.g_magic >> 16;
+      const int t = tok0 + tt;
+      const int hq = h * a.G + r - tt * a.G;
       __half* dst = a.out + (static_cast<size_t>(t) * a.Hq + hq) * 64;
 #pragma unroll
       for (int cch = 0; cch < 8; ++cch) {
@@ -625,6 +675,8 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
         *reinterpret_cast<uint4*>(dst + 8 * cch) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
       }
     }
+    __syncthreads();
+    free_tmem();
     return;
   }
 
@@ -653,11 +705,13 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
       put_row(stage + static_cast<size_t>(r % nitems) * blk_floats + (r / nitems) * kAttnRow);
     fence_proxy_async_smem();
     __syncthreads();
+    free_tmem();
     cluster_arrive_release();
     cluster_wait();   // every CTA of the cluster is done with its pages: receive buffers idle
     if (threadIdx.x == 0) {
       const uint32_t bytes = static_cast<uint32_t>(blk_floats * 4);
       const uint32_t dst_local = smem_u32(recv) + static_cast<uint32_t>(c) * bytes;
+#pragma unroll 1
       for (int q = 0; q < nitems; ++q)
         bulk_copy_to_peer(cluster_map(dst_local, static_cast<uint32_t>(q)),
                           smem_u32(stage) + static_cast<uint32_t>(q) * bytes, bytes,
@@ -669,9 +723,12 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
   } else {
     // ---- item rows -> global scratch; the last item to arrive merges
     if (row_thread) put_row(part_bh + (static_cast<size_t>(c) * rows_alloc + r) * kAttnRow);
-    __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) s_int[1] = (atomicAdd(a.ticket + bh, 1) == nitems - 1) ? 1 : 0;
+    free_tmem();
+    if (threadIdx.x == 0) {
+      __threadfence();   // behind the barrier: covers the rows every thread wrote
+      s_int[1] = (atomicAdd(a.ticket + bh, 1) == nitems - 1) ? 1 : 0;
+    }
     __syncthreads();
     if (!s_int[1]) return;
     __threadfence();
@@ -695,9 +752,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
   // ---- merge of items 0..nitems-1 in order for rows row_of(k), k < my_rows.
   //      mb/lb [item][k] hold m and l, then mb the coefficients w_it / L (one
   //      thread per row); then one thread per (row, 4 dims) sums coef * O_it.
-  //      Both live in the idle ring (in a cluster once this CTA's outgoing
-  //      copies have read it).
-  if (in_cluster && threadIdx.x == 0) bulk_wait_read_all();
+  if (in_cluster && threadIdx.x == 0) bulk_wait_read_all();   // outgoing rows have left
   __syncthreads();
   // cluster: the received rows fill the ring, the tables go over Q and P (the
   // outgoing copies have read them); global: the tables go in the ring
@@ -706,6 +761,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
   const bool fits = 2 * nitems * rows_alloc * 4 <= (in_cluster ? kAttnRingOff : kAttnRingBytes);
   if (!fits && threadIdx.x == 0) atomicExch(a.err, kErrBounds);
   if (fits) {
+#pragma unroll 1
     for (int idx = threadIdx.x; idx < nitems * my_rows; idx += blockDim.x) {
       const int it = idx / my_rows, k = idx - it * my_rows;
       const float2 ml = ld2(src_of(it, k) + 64);
@@ -715,10 +771,12 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
   }
   __syncthreads();
   if (fits) {
+#pragma unroll 1
     for (int k = threadIdx.x; k < my_rows; k += blockDim.x) {
       float M = -INFINITY;
       for (int it = 0; it < nitems; ++it) M = fmaxf(M, mb[it * rows_alloc + k]);
       float L = 0.f;
+#pragma unroll 1
       for (int it = 0; it < nitems; ++it) {
         const float mi = mb[it * rows_alloc + k];
         const float w = (mi == -INFINITY) ? 0.f : exp2f(mi - M);
@@ -726,14 +784,17 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
         L += w * lb[it * rows_alloc + k];
       }
       const float inv = 1.0f / L;
+#pragma unroll 1
       for (int it = 0; it < nitems; ++it) mb[it * rows_alloc + k] *= inv;
     }
   }
   __syncthreads();
   if (fits) {
+#pragma unroll 1
     for (int idx = threadIdx.x; idx < my_rows * 16; idx += blockDim.x) {
       const int k = idx >> 4, d4 = (idx & 15) * 4;
       float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
       for (int it0 = 0; it0 < nitems; it0 += 8) {   // 8 loads in flight, summed in order
         const int n8 = min(8, nitems - it0);
         float4 v[8];
@@ -752,8 +813,9 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
       }
       if (all_ok && got) {
         const int rr = row_of(k);
-        const int t = tok0 + rr / a.G;
-        const int hq = h * a.G + rr % a.G;
+        const int tt = rr * a.g_magic >> 16;
+        const int t = tok0 + tt;
+        const int hq = h * a.G + rr - tt * a.G;
         __half* dst = a.out + (static_cast<size_t>(t) * a.Hq + hq) * 64 + d4;
         *reinterpret_cast<__half2*>(dst) = __floats2half2_rn(acc.x, acc.y);
         *reinterpret_cast<__half2*>(dst + 2) = __floats2half2_rn(acc.z, acc.w);

@@ -378,7 +378,7 @@ size_t carve(gs_handle* h, const gs_config& c, void* base) {
   const int items_target =
       attn_use_cluster(kAttnMaxCluster, c.max_batch * g_dec.n_sub * c.n_kv_heads) ? kAttnMaxCluster : 8;
   int sp = c.split_pages > 0 ? c.split_pages : std::max(2, cdiv(pt_stride, items_target));
-  sp = std::max(sp, cdiv(pt_stride, attn_max_merge_items(g_dec.rows)));
+  sp = std::max(sp, cdiv(pt_stride, kAttnMaxMergeItems));
   const int items_dec = cdiv(pt_stride, sp);
   const int sp_pf = std::max(8, cdiv(pt_stride, 8));
   const int items_pf = cdiv(pt_stride, sp_pf);
@@ -562,6 +562,7 @@ int run_attention(gs_handle* h, int layer, int T, const AttnLaunch& L) {
   a.Hq = c.n_heads;
   a.Hkv = c.n_kv_heads;
   a.G = h->G;
+  a.g_magic = (65536 + h->G - 1) / h->G;
   a.rows_per_page = 2 * c.n_kv_heads * 64;
   a.kv_row_base = static_cast<long long>(layer) * h->n_pages * a.rows_per_page;
   a.split_pages = L.split_pages;
@@ -574,7 +575,7 @@ int run_attention(gs_handle* h, int layer, int T, const AttnLaunch& L) {
   if (!a.cluster &&
       (static_cast<size_t>(n_blocks) * c.n_kv_heads * L.max_items * g.rows * kAttnRow >
            h->attn_part_floats ||
-       L.max_items > attn_max_merge_items(g.rows)))
+       L.max_items > kAttnMaxMergeItems))
     return fail(h, GS_ERR_OOM, "attention item scratch too small");
   GS_CUDA(h, launch_attention(h->tm_kv, a, n_blocks, h->stream, h->pdl));
   note_launch(h, GS_KIND_ATTENTION);
@@ -1587,7 +1588,7 @@ int gs_attention(int mode, const void* q, const void* kv, int n_pages, const int
   if (ensure_kernel_attributes() != cudaSuccess) return GS_ERR_CUDA;
   const AttnGeom g = attn_geom(W, G);
   const int items = cdiv(pt_stride, split_pages);
-  if (items > attn_max_merge_items(g.rows)) return GS_ERR_UNSUPPORTED;
+  if (items > kAttnMaxMergeItems) return GS_ERR_UNSUPPORTED;
   const size_t blocks = static_cast<size_t>(n_seq) * g.n_sub;
   Carver cv(scratch);
   int* err = cv.take<int>(64);
@@ -1621,6 +1622,7 @@ int gs_attention(int mode, const void* q, const void* kv, int n_pages, const int
   a.Hq = n_heads;
   a.Hkv = n_kv_heads;
   a.G = G;
+  a.g_magic = (65536 + G - 1) / G;
   a.rows_per_page = 2 * n_kv_heads * 64;
   a.kv_row_base = 0;
   a.split_pages = split_pages;

@@ -55,16 +55,13 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
-// Wait for the phase with the given parity; false (and the error word set)
-// if it has not completed within limit_ns of %globaltimer.  The first try is
-// its own straight-line branch: try_wait itself suspends the thread until the
-// phase completes, so it nearly always succeeds there, and entering the retry
-// loop costs about 50 cycles per wait even when the phase is complete (a
-// 64-deep k-block of a TMA ring: 395 -> 300 cycles with both of its waits
-// written this way).
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* err,
-                                          uint64_t limit_ns = kWaitLimitNs) {
-  if (mbar_try_wait(bar, parity)) return true;
+// The retries of mbar_wait, bounded by limit_ns of %globaltimer.  Out of line:
+// every wait of a kernel shares this copy, so a pipeline's instructions stay in
+// the instruction cache (a kernel here runs for a few microseconds; one line
+// fetched from beyond the SM's cache costs a tenth of one, or more under load).
+static __device__ __noinline__ bool mbar_wait_retry(uint32_t bar, uint32_t parity, int* err,
+                                                    uint64_t limit_ns) {
+#pragma unroll 1
   for (int i = 0; i < 256; ++i)
     if (mbar_try_wait(bar, parity)) return true;
   const uint64_t t0 = global_timer_ns();
@@ -76,6 +73,18 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* er
     }
     __nanosleep(128);
   }
+}
+
+// Wait for the phase with the given parity; false (and the error word set)
+// if it has not completed within limit_ns of %globaltimer.  try_wait itself
+// suspends the thread until the phase completes, so the first try nearly
+// always succeeds; entering a retry loop for it costs about 50 cycles per wait
+// (a 64-deep k-block of a TMA ring: 395 -> 300 cycles with its two waits
+// written this way).
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* err,
+                                          uint64_t limit_ns = kWaitLimitNs) {
+  if (mbar_try_wait(bar, parity)) return true;
+  return mbar_wait_retry(bar, parity, err, limit_ns);
 }
 
 // Position in a ring of `n` stages: the stage and the parity of its use,
