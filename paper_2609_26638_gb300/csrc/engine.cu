@@ -60,6 +60,19 @@ bool gs::make_map(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols
   return r == CUDA_SUCCESS;
 }
 
+bool gs::make_map_swiglu(CUtensorMap* m, const void* base, uint64_t N, uint64_t K) {
+  EncodeTiledFn enc = get_encode();
+  if (!enc) return false;
+  cuuint64_t dims[4] = {K, 16, 2, N / 16};
+  cuuint64_t strides[3] = {K * 2, N * K * 2, 16 * K * 2};
+  cuuint32_t box[4] = {64, 16, 2, 4};
+  cuuint32_t es[4] = {1, 1, 1, 1};
+  CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<void*>(base), dims, strides,
+                   box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS;
+}
+
 namespace {
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -153,37 +166,24 @@ int decode_splits(int weight_rows, int K) {
   return s;
 }
 
-// Decode windows of up to 64 tokens split K across the CTAs of a cluster.
-// Wider decode launches with at least 8 k-blocks per split keep that (64-token
-// tiles); the others reduce the same K chunks inside each CTA
-// (gemm_chunk_kernel: each chunk summed from zero in a TMEM buffer, then added
-// in chunk order to a running sum in TMEM), with the token tile the widest of
-// 128 / 64 / 32 with the fewest waves x operand bytes per CTA.  All three
-// give the same sums in the same order.  Prefill does not split K.
+// Decode windows of up to 64 tokens split K across the CTAs of a cluster: one
+// or two token tiles of few feature tiles would leave most SMs idle.  Wider
+// launches reduce the same K chunks inside each CTA of the persistent kernel
+// (each chunk summed from zero in a TMEM buffer, the chunks added in order), as
+// does every launch that is not split.  The sums and their order are the same.
+// Measured at 544 rows: down projection 22.5 us in clusters of 8 with 64-token
+// tiles, see the persistent kernel's header for its side.
 GemmPlan plan_split(int weight_rows, int T, int S, int nkb) {
   GemmPlan p;
   p.feat_tiles = weight_rows / 128;
-  p.chunks = 1;
-  p.splits = S;
-  p.bn = gemm_bn_for(T);
-  if (S > 1 && T > 64 && nkb / S >= 8 && gemm_cluster_ok(64, S)) {
-    p.bn = 64;
-  } else if (S > 1 && T > 64) {
-    // chunked K inside each CTA (gemm_chunk_kernel, two CTAs per SM).  A CTA
-    // streams K x (128 + BN) operand bytes, and the launch takes ceil(CTAs /
-    // slots) rounds of them: pick the token tile of 128 / 64 / 32 with the
-    // least waves x (128 + BN), the wider on a tie.
-    p.chunks = S;
+  if (S > 1 && T <= 64) {
+    p.splits = S;
+    p.chunks = 1;
+    p.bn = T <= 32 ? 32 : 64;
+  } else {
     p.splits = 1;
-    long best = -1;
-    for (int bn : {128, 64, 32}) {
-      const long waves = cdiv(static_cast<long long>(p.feat_tiles) * cdiv(T, bn), 2 * kNumSMs);
-      const long cost = waves * (128 + bn);
-      if (best < 0 || cost < best) {
-        best = cost;
-        p.bn = bn;
-      }
-    }
+    p.chunks = S;
+    p.bn = wide_bn(p.feat_tiles, T, nkb);
   }
   p.tok_tiles = cdiv(T, p.bn);
   return p;
@@ -227,7 +227,7 @@ struct gs_handle {
   __half* wcopy = nullptr;
   std::vector<CUtensorMap> tm_qkv, tm_o, tm_gu, tm_down;
   CUtensorMap tm_lm;
-  CUtensorMap tm_hb[4], tm_ao[4], tm_act[4];
+  CUtensorMap tm_hb[kWideTiles], tm_ao[kWideTiles], tm_act[kWideTiles];
   CUtensorMap tm_kv;
 
   // sizes
@@ -334,8 +334,6 @@ void note_launch(gs_handle* h, int kind) {
   if (r != cudaSuccess && h->prof_err == cudaSuccess) h->prof_err = r;
   h->prof_kind.push_back(kind);
 }
-
-int bn_index(int bn) { return bn == 32 ? 0 : (bn == 64 ? 1 : (bn == 128 ? 2 : 3)); }
 
 bool config_ok(const gs_config* c, std::string* why) {
   auto bad = [&](const char* m) { *why = m; return false; };
@@ -530,7 +528,7 @@ int run_gemm(gs_handle* h, const CUtensorMap& tw, int weight_rows, const CUtenso
       (static_cast<size_t>(p.splits) * p.feat_tiles * p.tok_tiles * p.bn * 128 > h->partial_floats ||
        p.feat_tiles * p.tok_tiles > kGemmCounters))
     return fail(h, GS_ERR_OOM, "split-K scratch too small");
-  GS_CUDA(h, launch_gemm(p.bn, epi, tw, tx_set[bn_index(p.bn)], a, p.feat_tiles, p.tok_tiles,
+  GS_CUDA(h, launch_gemm(p.bn, epi, tw, tx_set[wide_index(p.bn)], a, p.feat_tiles, p.tok_tiles,
                          h->stream, h->pdl));
   note_launch(h, kind);
   return GS_OK;
@@ -1103,14 +1101,13 @@ int gs_create(const gs_config* cfg, const gs_weights* w, void* workspace, size_t
   for (int l = 0; l < L && ok; ++l)
     ok = make_map(&h->tm_qkv[l], h->w_qkv[l], h->qkv_dim, d, 128) &&
          make_map(&h->tm_o[l], h->w_o[l], d, HD, 128) &&
-         make_map(&h->tm_gu[l], h->w_gu[l], 2 * F, d, 64) &&
+         make_map_swiglu(&h->tm_gu[l], h->w_gu[l], F, d) &&
          make_map(&h->tm_down[l], h->w_down[l], d, F, 128);
   ok = ok && make_map(&h->tm_lm, h->lm_head, c.vocab, d, 128);
-  const int bns[4] = {32, 64, 128, 256};
-  for (int i = 0; i < 4 && ok; ++i) {
-    ok = make_map(&h->tm_hb[i], h->hb, h->T_max, d, bns[i]) &&
-         make_map(&h->tm_ao[i], h->ao, h->T_max, HD, bns[i]) &&
-         make_map(&h->tm_act[i], h->act, h->T_max, F, bns[i]);
+  for (int i = 0; i < kWideTiles && ok; ++i) {
+    ok = make_map(&h->tm_hb[i], h->hb, h->T_max, d, kWideBN[i]) &&
+         make_map(&h->tm_ao[i], h->ao, h->T_max, HD, kWideBN[i]) &&
+         make_map(&h->tm_act[i], h->act, h->T_max, F, kWideBN[i]);
   }
   const uint64_t kv_rows = static_cast<uint64_t>(L) * h->n_pages * 2 * c.n_kv_heads * 64;
   ok = ok && kv_rows < (1ull << 31) && make_map(&h->tm_kv, h->kv, kv_rows, 64, 64);
@@ -1637,16 +1634,17 @@ int gs_attention(int mode, const void* q, const void* kv, int n_pages, const int
 
 size_t gs_linear_scratch_bytes(int M, int N, int split_k) {
   if (M < 1 || N < 64 || split_k < 1) return 0;
-  // the larger of the plans for an N-row and a 2N-row (SwiGLU) weight
+  // the larger of the plans for an N-row and a 2N-row (SwiGLU) weight; only a
+  // launch that splits K across CTAs needs counters (and partials, unless its
+  // CTAs form clusters), and its tiles do not depend on K
   size_t counters = 0, partial = 0;
   for (int w_rows : {N, 2 * N}) {
-    for (int nkb : {split_k, 8 * split_k}) {   // the plans for short and long K per split
-      const GemmPlan p = plan_split(w_rows, M, split_k, nkb);
-      counters = std::max(counters, static_cast<size_t>(p.tok_tiles) * p.feat_tiles);
-      if (p.splits > 1 && !gemm_cluster_ok(p.bn, p.splits))
-        partial = std::max(partial, static_cast<size_t>(p.splits) * p.tok_tiles * p.feat_tiles *
-                                        p.bn * 128);
-    }
+    const GemmPlan p = plan_split(w_rows, M, split_k, split_k);
+    if (p.splits == 1) continue;
+    counters = std::max(counters, static_cast<size_t>(p.tok_tiles) * p.feat_tiles);
+    if (!gemm_cluster_ok(p.bn, p.splits))
+      partial = std::max(partial, static_cast<size_t>(p.splits) * p.tok_tiles * p.feat_tiles *
+                                      p.bn * 128);
   }
   Carver cv(nullptr);
   cv.take<int>(64);
@@ -1668,18 +1666,19 @@ int gs_linear(const void* x, const void* w, void* y, int M, int N, int K, int ep
       (reinterpret_cast<uintptr_t>(y) & 15))
     return GS_ERR_INVALID_ARG;
   if (ensure_kernel_attributes() != cudaSuccess) return GS_ERR_CUDA;
-  // split-K as the decoder plans it: across the CTAs of a cluster (up to 64
-  // rows), as chunks inside each CTA (wider), else through global scratch
+  // split-K as the decoder plans it: across the CTAs of a cluster or through
+  // global scratch (up to 64 rows), as chunks inside each CTA (wider)
   const int w_rows = epilogue == kEpiSwiGLU ? 2 * N : N;
   const GemmPlan p = plan_split(w_rows, M, split_k, K / 64);
   const int bn = p.bn, tok_tiles = p.tok_tiles, feat_tiles = p.feat_tiles;
   CUtensorMap tw, tx;
-  if (!make_map(&tw, w, w_rows, K, epilogue == kEpiSwiGLU ? 64 : 128)) return GS_ERR_INVALID_ARG;
+  if (!(epilogue == kEpiSwiGLU ? make_map_swiglu(&tw, w, N, K) : make_map(&tw, w, w_rows, K, 128)))
+    return GS_ERR_INVALID_ARG;
   if (!make_map(&tx, x, M, K, bn)) return GS_ERR_INVALID_ARG;
   Carver cv(scratch);
   GemmArgs a = {};
   a.err = cv.take<int>(64);
-  a.counters = cv.take<int>(static_cast<size_t>(tok_tiles) * feat_tiles);
+  if (p.splits > 1) a.counters = cv.take<int>(static_cast<size_t>(tok_tiles) * feat_tiles);
   // The error word and the per-tile arrival counters of the global split-K
   // path must start at zero, whatever the caller's scratch held before.
   const size_t head_bytes = cv.off;
@@ -1698,8 +1697,8 @@ int gs_linear(const void* x, const void* w, void* y, int M, int N, int K, int ep
   a.logits = nullptr;
   a.w_scale = 1.f;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(scratch, 0, head_bytes, s) != cudaSuccess) return GS_ERR_CUDA;
-  return launch_gemm(bn, epilogue, tw, tx, a, feat_tiles, tok_tiles, s) == cudaSuccess
+  if (clear_words(static_cast<int*>(scratch), head_bytes / 4, s) != cudaSuccess) return GS_ERR_CUDA;
+  return launch_gemm(bn, epilogue, tw, tx, a, feat_tiles, tok_tiles, s, true) == cudaSuccess
              ? GS_OK
              : GS_ERR_CUDA;
 }

@@ -60,19 +60,70 @@ inline bool gemm_cluster_ok(int bn, int splits) {
   const int per = bn / splits;
   return per <= 8 || 32 % per == 0;
 }
+// Token tiles of the persistent GEMM (splits == 1) and, per 64-deep k-block of
+// one, the cycles its ring takes with one CTA per SM (measured: 240 / 257 / 290
+// cycles at 32 / 64 / 96 rows, where L2 -> shared memory bounds it, 350 / 410 /
+// 515 at 144 / 192 / 256, towards the MMA rate of 2 cycles per row).
+constexpr int kWideTiles = 6;
+constexpr int kWideBN[kWideTiles] = {32, 64, 96, 144, 192, 256};
+constexpr int kWideCycles[kWideTiles] = {240, 257, 290, 350, 410, 515};
+
+inline int wide_index(int bn) {
+  for (int i = 0; i < kWideTiles; ++i)
+    if (kWideBN[i] == bn) return i;
+  return -1;
+}
+
+// The token tile with the least estimated time: rounds of tiles over the SMs,
+// each the longer of its k-blocks and its epilogue slices (about 700 cycles per
+// 32 tokens of a group; one group of warps at 32 rows, else two), and the last
+// tile's epilogue, which nothing overlaps.  The wider on a tie.
+inline int wide_bn(int feat_tiles, int T, int nkb) {
+  int best = 32;
+  long long best_cost = -1;
+  for (int i = kWideTiles - 1; i >= 0; --i) {
+    const int bn = kWideBN[i];
+    const long long tiles = static_cast<long long>(feat_tiles) * ((T + bn - 1) / bn);
+    const long long rounds = (tiles + kNumSMs - 1) / kNumSMs;
+    const long long main = static_cast<long long>(nkb) * kWideCycles[i];
+    const long long epi = 700ll * ((bn / (bn >= 64 ? 2 : 1) + 31) / 32);
+    const long long cost = rounds * (main > epi ? main : epi) + epi;
+    if (best_cost < 0 || cost < best_cost) {
+      best_cost = cost;
+      best = bn;
+    }
+  }
+  return best;
+}
+
 cudaError_t launch_gemm(int bn, int epi, const CUtensorMap& tmW, const CUtensorMap& tmX,
                         const GemmArgs& args, int feat_tiles, int tok_tiles, cudaStream_t s,
                         bool pdl = false);
+
+// Zero n words on the stream with a kernel that lets a dependent launch (PDL)
+// start its prologue at once: a launch after it costs about 3 us less than after
+// a memset node, whose completion the next kernel's launch waits for.
+cudaError_t clear_words(int* p, size_t n, cudaStream_t s);
+
+// The persistent kernel (args.splits == 1, bn one of kWideBN).
+cudaError_t launch_gemm_wide(int bn, int epi, const CUtensorMap& tmW, const CUtensorMap& tmX,
+                             const GemmArgs& args, int feat_tiles, int tok_tiles, cudaStream_t s,
+                             bool pdl);
 
 // 2-D fp16 tensor map over a row-major [rows, cols] array, box {64 columns,
 // box_rows rows}, 128-byte swizzle, zero fill out of bounds.  The driver's
 // encoder is looked up once per process (thread-safe).  False if the lookup
 // or the encode fails.
 bool make_map(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows);
-
+// The map of a SwiGLU weight [2 N, K] (gate rows, then up rows): one box holds
+// the 128 rows of 64 output features in four groups of 16 gate rows and their
+// 16 up rows, so the two rows of a feature land in one warp's TMEM lanes.
+// N % 64 == 0.
+bool make_map_swiglu(CUtensorMap* m, const void* base, uint64_t N, uint64_t K);
 
 // Sets the dynamic shared-memory limit of every GEMM instantiation once.
 cudaError_t gemm_init_attributes();
+cudaError_t gemm_wide_init_attributes();
 // Every kernel's launch attributes on the current device, once per device
 // (thread-safe); call before the first launch.
 cudaError_t ensure_kernel_attributes();

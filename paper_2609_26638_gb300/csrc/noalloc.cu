@@ -78,9 +78,13 @@ extern "C" int gs_linear_noalloc(const void* x, const void* w, void* y, int M, i
   void* base = nullptr;
   int rc = scratch_for_current_device(&base);
   if (rc != GS_OK) return rc;
+  // unsplit launches run on the persistent kernel's token tiles
+  const int run_bn = split_k == 1 ? wide_bn(feat_tiles, M, K / 64) : bn;
+  const int run_tok_tiles = (M + run_bn - 1) / run_bn;
   CUtensorMap tw, tx;
-  if (!make_map(&tw, w, w_rows, K, epilogue == kEpiSwiGLU ? 64 : 128)) return GS_ERR_INVALID_ARG;
-  if (!make_map(&tx, x, M, K, bn)) return GS_ERR_INVALID_ARG;
+  if (!(epilogue == kEpiSwiGLU ? make_map_swiglu(&tw, w, N, K) : make_map(&tw, w, w_rows, K, 128)))
+    return GS_ERR_INVALID_ARG;
+  if (!make_map(&tx, x, M, K, run_bn)) return GS_ERR_INVALID_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   uint8_t* b = static_cast<uint8_t*>(base);
   // the split-K counters must start at zero; the array keeps the last call's contents
@@ -94,13 +98,15 @@ extern "C" int gs_linear_noalloc(const void* x, const void* w, void* y, int M, i
   a.K = K;
   a.splits = split_k;
   a.cluster = 0;
+  a.chunks = 1;
   a.kb_per_split = (K / 64) / split_k;
   a.y = y;
   a.ldy = N;
   a.logits = nullptr;
   a.w_scale = 1.f;
-  return launch_gemm(bn, epilogue, tw, tx, a, feat_tiles, tok_tiles, s) == cudaSuccess ? GS_OK
-                                                                                        : GS_ERR_CUDA;
+  return launch_gemm(run_bn, epilogue, tw, tx, a, feat_tiles, run_tok_tiles, s) == cudaSuccess
+             ? GS_OK
+             : GS_ERR_CUDA;
 }
 
 extern "C" int gs_linear_noalloc_status(void* stream) {

@@ -144,6 +144,16 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* m, 
       : "memory");
 }
 
+// The 4-D form (coordinates innermost first; x as above).
+__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* m, int x, int y, int z,
+                                            int w, uint32_t bar, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1, {%2, %3, %4, %5}], [%6], %7;" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar), "l"(policy)
+      : "memory");
+}
+
 // ---------------------------------------------------------------- tcgen05
 __device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem),
@@ -347,6 +357,34 @@ __device__ __forceinline__ const float* cluster_peer_ptr(const float* p, uint32_
   uint64_t g;
   asm volatile("mapa.u64 %0, %1, %2;" : "=l"(g) : "l"(reinterpret_cast<uint64_t>(p)), "r"(rank));
   return reinterpret_cast<const float*>(g);
+}
+
+// ---------------------------------------------------------------- cluster launch control
+// Ask the hardware for a CTA of this grid that has not started: the 16-byte
+// answer lands in shared memory and completes 16 bytes on `bar`.
+__device__ __forceinline__ void clc_try_cancel(uint32_t slot, uint32_t bar) {
+  asm volatile(
+      "clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
+      ::"r"(slot), "r"(bar)
+      : "memory");
+}
+// True and that CTA's index, or false: every CTA has started.
+__device__ __forceinline__ bool clc_answer(uint32_t slot, int* x, int* y, int* z) {
+  uint32_t ok, cx = 0, cy = 0, cz = 0;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b128 h;\n\t"
+      "ld.shared.b128 h, [%4];\n\t"
+      "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, h;\n\t"
+      "selp.u32 %3, 1, 0, p;\n\t"
+      "mov.u32 %0, 0;\n\tmov.u32 %1, 0;\n\tmov.u32 %2, 0;\n\t"
+      "@p clusterlaunchcontrol.query_cancel.get_first_ctaid.v4.b32.b128 {%0, %1, %2, _}, h;\n\t}"
+      : "=r"(cx), "=r"(cy), "=r"(cz), "=r"(ok)
+      : "r"(slot)
+      : "memory");
+  *x = static_cast<int>(cx);
+  *y = static_cast<int>(cy);
+  *z = static_cast<int>(cz);
+  return ok != 0;
 }
 
 // ---------------------------------------------------------------- fp16 stores

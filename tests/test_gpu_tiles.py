@@ -1,0 +1,74 @@
+"""GPU parity at the edges of the persistent GEMM's tiles: token tiles of 32 to 256
+rows and their remainders, odd k-block counts, in-CTA K chunks, the resident
+token tile, SwiGLU gates outside the fast quotient's range.
+
+References and tolerances as in test_gpu_kernels.py (fp32 matmul of the same
+fp16 operands, 2^-11 relative for fp16 stores)."""
+import pytest
+import torch
+
+from tests.test_gpu_kernels import DEV, _linear
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gs():
+    from paper_2609_26638_gb300 import gs as binding
+    return binding
+
+
+@pytest.mark.parametrize("M,N,K,split", [
+    (1, 128, 64, 1), (65, 256, 64, 1), (96, 384, 192, 3), (97, 2048, 1024, 8), (144, 1024, 704, 1),
+    (145, 1024, 4096, 8), (192, 8192, 320, 1), (193, 2048, 640, 5), (256, 20480, 128, 2),
+    (257, 4096, 192, 1), (1000, 1024, 1024, 16),
+])
+def test_linear_tile_edges(gs, M, N, K, split):
+    g = torch.Generator(device=DEV).manual_seed(M + N + K)
+    x = torch.randn(M, K, device=DEV, generator=g).half()
+    w = (0.02 * torch.randn(N, K, device=DEV, generator=g)).half()
+    ref = x.float() @ w.float().T
+    y = torch.zeros(M, N, dtype=torch.float16, device=DEV)
+    _linear(gs, x, w, M, N, K, gs.EPI_STORE_F16, split, y)
+    torch.testing.assert_close(y.float(), ref, rtol=2e-3, atol=1e-3 * ref.abs().max().item())
+    base = torch.randn(M, N, device=DEV, generator=g)
+    r = base.clone()
+    _linear(gs, x, w, M, N, K, gs.EPI_RESID_F32, split, r)
+    torch.testing.assert_close(r, base + ref, rtol=1e-4, atol=1e-4 * ref.abs().max().item())
+
+
+@pytest.mark.parametrize("M", [1, 32, 33, 300])
+@pytest.mark.parametrize("K", [64, 960, 1024, 2048])
+def test_linear_argmax_more_tiles_than_sms(gs, M, K):
+    """153 feature tiles: with at most 32 rows and K <= 1024 the token tile stays
+    resident.  The returned row is the reference's, or within the fp32 summation
+    error of its value (K products of N(0, 1) x 0.02 N(0, 1), 2^-24 each)."""
+    V = 153 * 128
+    g = torch.Generator(device=DEV).manual_seed(M * 3 + K)
+    x = torch.randn(M, K, device=DEV, generator=g).half()
+    w = (0.02 * torch.randn(V, K, device=DEV, generator=g)).half()
+    ref = x.double() @ w.double().T
+    keys = torch.zeros(M, dtype=torch.int64, device=DEV)
+    _linear(gs, x, w, M, V, K, gs.EPI_ARGMAX, 1, keys)
+    idx = 0xFFFFFFFF - (keys & 0xFFFFFFFF)
+    got = ref.gather(1, idx[:, None])[:, 0]
+    assert bool((ref.max(dim=1).values - got <= 1e-4).all())
+
+
+@pytest.mark.parametrize("M,split", [(3, 1), (40, 2), (200, 1)])
+def test_swiglu_gates_of_any_size(gs, M, split):
+    """Gates from about -300 to 300: exp overflows on the negative side (silu is
+    then -0), and rows of zeros keep zero."""
+    F, K = 512, 256
+    g = torch.Generator(device=DEV).manual_seed(9 + M)
+    x = torch.randn(M, K, device=DEV, generator=g).half()
+    x[M // 2] = 0
+    wg = torch.randn(F, K, device=DEV, generator=g) * 5.0
+    wu = torch.randn(F, K, device=DEV, generator=g) * 0.02
+    w = torch.cat([wg, wu]).half()
+    gu = x.double() @ w.double().T
+    ref = gu[:, :F] * torch.sigmoid(gu[:, :F]) * gu[:, F:]
+    y = torch.full((M, F), 7.0, dtype=torch.float16, device=DEV)
+    _linear(gs, x, w, M, F, K, gs.EPI_SWIGLU, split, y)
+    torch.testing.assert_close(y.double(), ref, rtol=2e-3, atol=1e-3)
+    assert float(y[M // 2].abs().max()) == 0.0
