@@ -32,13 +32,15 @@
 //
 // Merge over items, item order 0, 1, ...: M = max m_i, w_i = exp2(m_i - M),
 // coef_i = w_i / sum_j w_j l_j, O = sum coef_i O_i.  A block with one item
-// writes its rows directly.  A (block, head) with at most 16 items may form one
-// thread-block cluster: once every CTA of the cluster has finished its pages,
-// each sends the rows that CTA (r mod n) owns to it with one bulk async copy
-// into its shared memory, completing on its mbarrier, and each owner merges
-// its rows.  Otherwise every item writes its rows to global scratch and the
-// last one to finish (atomic ticket per (block, head), no spinning) merges
-// them.  Both paths run the same arithmetic in the same order.
+// writes its rows directly.  The kernel of this file is for small launches (at
+// most 16 items per (block, head), about one wave of CTAs): the items of a
+// (block, head) form a thread-block cluster, and once every CTA of it has
+// finished its pages, each sends the rows that CTA (r mod n) owns to it with one
+// bulk async copy into its shared memory, completing on its mbarrier, and each
+// owner merges its rows.  Larger launches run attention_stream.cuh: there every
+// item writes its rows to global scratch and the last one to finish (atomic
+// ticket per (block, head), no spinning) merges them.  Both run the same
+// arithmetic in the same order.
 //
 // Invariance.  Item boundaries are absolute page numbers fixed by SP, pages
 // are reduced in order, the MMA's arithmetic for a row does not depend on the
@@ -74,7 +76,7 @@ constexpr int kAttnKRingBytes = kAttnKStages * kAttnPageBytes;
 constexpr int kAttnRingBytes = kAttnKRingBytes + kAttnVStages * kAttnVStageBytes;
 // Q [128][128 B] | P[2] [128][128 B] | K ring | V^T ring | barriers.  After the
 // pages are done, Q and P hold the owner-grouped rows (cluster) and the rings
-// the received rows or the merge's (m, l) tables.
+// the received rows.
 constexpr int kAttnQOff = 0;
 constexpr int kAttnPOff = kAttnMaxRows * 128;
 constexpr int kAttnRingOff = kAttnPOff + 2 * kAttnMaxRows * 128;
@@ -83,11 +85,8 @@ constexpr int kAttnSmemBytes = 1024 + kAttnBarOff + 256 + kAttnMaxRows * 4 + kAt
 constexpr int kAttnRowsFloats = (kAttnMaxRows + kAttnMaxCluster) * kAttnRow;
 static_assert(kAttnRingOff >= kAttnRowsFloats * 4 && kAttnRingBytes >= kAttnRowsFloats * 4,
               "Q + P hold the owner-grouped rows, the ring the received rows");
-static_assert(kAttnRingOff >= 2 * kAttnMaxCluster * kAttnMaxRows * 4, "Q + P hold a cluster's tables");
-// Items one global merge takes (an interface limit: the tables of m and l, 1 KB
-// per item, have to fit the ring).
+// Items one merge through global scratch takes (an interface limit).
 constexpr int kAttnMaxMergeItems = 54;
-static_assert(kAttnMaxMergeItems * 2 * kAttnMaxRows * 4 <= kAttnRingBytes, "merge tables");
 
 struct AttnArgs {
   const __half* q;            // [T, Hq, 64]
@@ -107,7 +106,8 @@ struct AttnArgs {
   int rows_per_page;          // 2 * Hkv * 64
   int split_pages;            // SP: pages per item
   int max_items;              // items per (block, head) the grid covers
-  int cluster;                // 1: the grid's x dimension is one cluster (max_items <= 16)
+  int cluster;                // 1: the grid's x dimension is one cluster (max_items <= 16), attn_paged_kernel
+  int early;                  // 1: the launch before this one does not write the descriptors or limits
   float* part;                // global merge: [n_blocks][Hkv][max_items][128][kAttnRow]
   int* ticket;                // global merge: [n_blocks][Hkv], zero between launches
   int* err;
@@ -178,6 +178,43 @@ struct AttnSync {
 // MMA row (TMEM lane) -> block row, and back.
 __device__ __forceinline__ int attn_block_row(int mrow) { return (mrow & 31) * 4 + (mrow >> 5); }
 
+// Key limits of the rows a thread shares: set q (rows 8 q + lane / 4 of the
+// quarter), -1 past the block's rows.
+__device__ __forceinline__ void attn_row_limits(const AttnArgs& a, int warp, int R, int tok0,
+                                                int (&lim)[4]) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int rr = (8 * q + ((threadIdx.x & 31) >> 2)) * 4 + warp;
+    lim[q] = rr < R ? a.lim[tok0 + (rr * a.g_magic >> 16)] : -1;
+  }
+}
+
+// This thread's 8 of the 1,024 16-byte pieces of the block's Q rows (MMA row i
+// holds block row attn_block_row(i), zero past R), all loads in flight
+// together; then into the swizzled Q tile (rows past the last set are not read).
+__device__ __forceinline__ void attn_load_q(const AttnArgs& a, int h, int tok0, int R, uint4 (&v)[8]) {
+  const int ch = threadIdx.x & 7, i0 = threadIdx.x >> 3;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int rr = attn_block_row(i0 + 16 * k);
+    v[k] = make_uint4(0, 0, 0, 0);
+    if (rr < R) {
+      const int tt = rr * a.g_magic >> 16;
+      const int hq = h * a.G + rr - tt * a.G;
+      v[k] = *reinterpret_cast<const uint4*>(a.q + (static_cast<size_t>(tok0 + tt) * a.Hq + hq) * 64 + ch * 8);
+    }
+  }
+}
+__device__ __forceinline__ void attn_store_q(uint8_t* sQ, int R, const uint4 (&v)[8]) {
+  const int ch = threadIdx.x & 7, i0 = threadIdx.x >> 3;
+  const int lanes_used = ((R + 3) / 4 + 7) / 8 * 8;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int i = i0 + 16 * k;
+    if ((i & 31) < lanes_used) *reinterpret_cast<uint4*>(sQ + sw128(i, ch)) = v[k];
+  }
+}
+
 // Online softmax over the item's pages for one warp and the rows of its lane
 // quarter.  S comes from TMEM in the 16x256b layout, so a row is spread over
 // four neighbouring threads and a set of 8 rows costs a thread 16 columns,
@@ -197,21 +234,21 @@ __device__ __forceinline__ int attn_block_row(int mrow) { return (mrow & 31) * 4
 // unrolled variants this replaces spent 10 k of a CTA's 34 k cycles on that.
 // Waits are bounded; a warp whose wait ran out keeps arriving on the MMA
 // warp's barriers to the last page.  Returns false if a wait ran out.
+struct AttnRings {
+  RingPos s;   // S / P buffer of the next page
+  RingPos v;   // V^T ring stage of the next page
+};
+
 __device__ __forceinline__ bool attn_softmax(const AttnArgs& a, const AttnSync& y, uint32_t tmem,
-                                             int warp, int rows_w, int np, int p_begin, int R,
-                                             int tok0) {
+                                             int warp, int nset, int np, int p_begin,
+                                             const int (&lim)[4], AttnRings& rg) {
   const int lane = threadIdx.x & 31;
   const int quad = lane & 3;
-  const int nset = (rows_w + 7) / 8;   // sets of 8 rows, two per half
   float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-  int lim[4];
   int full_lim = 0x7FFFFFFF;   // every row of the warp sees the keys up to here
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int rr = (8 * q + (lane >> 2)) * 4 + warp;
-    lim[q] = rr < R ? a.lim[tok0 + (rr * a.g_magic >> 16)] : -1;
-    if (rr < R) full_lim = min(full_lim, lim[q]);
-  }
+  for (int q = 0; q < 4; ++q)
+    if (lim[q] >= 0) full_lim = min(full_lim, lim[q]);
   full_lim = __reduce_min_sync(0xFFFFFFFFu, full_lim);
   const uint32_t trow = tmem + (static_cast<uint32_t>(warp * 32) << 16);
   // row (warp * 32 + lane / 4) of the P tile; chunk j of row r sits at (j ^ (r & 7)) * 16
@@ -224,12 +261,12 @@ __device__ __forceinline__ bool attn_softmax(const AttnArgs& a, const AttnSync& 
     if (ok) ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, a.err)) != 0;
     return ok;
   };
-  RingPos prev;   // V^T ring position of page j - 1
+  RingPos prev;          // V^T ring stage of page j - 1
   bool pv_seen = true;   // O += P V of page j - 1 is known to have retired
 #pragma unroll 1
   for (int j = 0; j < np; ++j) {
-    const int buf = j & 1;
-    const bool have = wwait(s_full0 + 8 * buf, (j >> 1) & 1);
+    const int buf = rg.s.s;
+    const bool have = wwait(s_full0 + 8 * buf, rg.s.ph);
     const int key0 = (p_begin + j) * 64;
     if (have) {
       tc_fence_after();
@@ -323,13 +360,14 @@ __device__ __forceinline__ bool attn_softmax(const AttnArgs& a, const AttnSync& 
         if (two) put(1, mh[1], prow + 8 * 128);
       }
       fence_proxy_async_smem();
-    } else if (lane == 0) {
-      mbar_arrive(s_free0 + 8 * buf);
     }
+    if ((!have || nset == 0) && lane == 0) mbar_arrive(s_free0 + 8 * buf);
     tc_fence_before();
     __syncwarp();
     if (lane == 0) mbar_arrive(p_full0 + 8 * buf);
-    if (j > 0) prev.next(kAttnVStages);
+    prev = rg.v;
+    rg.v.next(kAttnVStages);
+    rg.s.next(2);
     pv_seen = false;
   }
   if (quad == 0) {
@@ -380,11 +418,11 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
   const int ntok = min(min(a.QS, a.QB - sub * a.QS), a.T - tok0);
   if (ntok <= 0) return;
   const int R = ntok * a.G;
-  const int nbusy = min(R, kAttnSoftWarps);   // softmax warps with rows
 
   // One round of global latency: warp 0 reads the block's descriptors while
   // the others set up barriers, TMEM and the ones rows.
   if (warp == 0) {
+    if (!a.early) pdl_wait();
     const int act = a.blk_active != nullptr ? a.blk_active[seq] : 1;
     const int sl = a.blk_slot ? a.blk_slot[seq] : a.fixed_slot;
     int lm[4];   // ntok <= 128
@@ -401,8 +439,8 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
       for (int s = 0; s < 2 * (kAttnKStages + kAttnVStages); ++s) mbar_init(smem_u32(&bars[s]), 1);
       for (int i = 0; i < 2; ++i) {
         mbar_init(smem_u32(&s_full[i]), 1);
-        mbar_init(smem_u32(&s_free[i]), nbusy);   // one arrival per softmax warp with rows
-        mbar_init(smem_u32(&p_full[i]), nbusy);
+        mbar_init(smem_u32(&s_free[i]), kAttnSoftWarps);   // one arrival per softmax warp
+        mbar_init(smem_u32(&p_full[i]), kAttnSoftWarps);
       }
       mbar_init(smem_u32(mma_done), 1);
       mbar_init(smem_u32(q_full), kAttnSoftWarps);
@@ -581,33 +619,20 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
   } else {
     // ---- softmax warps: Q rows -> swizzled smem (MMA row i holds block row
     // attn_block_row(i), zero past R; rows past the last set are not read)
-    const int rows_w = warp < nbusy ? (R - warp + 3) / 4 : 0;   // rows in this warp's quarter
-    const int lanes_used = ((R + 3) / 4 + 7) / 8 * 8;
+    const int rows_w = warp < R ? (R - warp + 3) / 4 : 0;   // rows in this warp's quarter
     pdl_wait();
     pdl_trigger();
-    const int ch = threadIdx.x & 7, i0 = threadIdx.x >> 3;
     uint4 v[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {   // all loads in flight together
-      const int i = i0 + 16 * k, rr = attn_block_row(i);
-      v[k] = make_uint4(0, 0, 0, 0);
-      if (rr < R) {
-        const int tt = rr * a.g_magic >> 16;
-        const int t = tok0 + tt;
-        const int hq = h * a.G + rr - tt * a.G;
-        v[k] = *reinterpret_cast<const uint4*>(a.q + (static_cast<size_t>(t) * a.Hq + hq) * 64 + ch * 8);
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int i = i0 + 16 * k;
-      if ((i & 31) < lanes_used) *reinterpret_cast<uint4*>(sQ + sw128(i, ch)) = v[k];
-    }
+    attn_load_q(a, h, tok0, R, v);
+    attn_store_q(sQ, R, v);
     fence_proxy_async_smem();
     __syncwarp();
     if (lane == 0) mbar_arrive(smem_u32(q_full));
     AttnSync y{s_full, s_free, p_full, v_empty, sP, m_row};
-    if (rows_w > 0) ok = attn_softmax(a, y, tmem, warp, rows_w, np, p_begin, R, tok0);
+    int lim[4];
+    attn_row_limits(a, warp, R, tok0, lim);
+    AttnRings rg;
+    ok = attn_softmax(a, y, tmem, warp, (rows_w + 7) / 8, np, p_begin, lim, rg);
   }
 
   // every MMA retired and every TMA copy landed before TMEM and the ring are reused
@@ -688,140 +713,70 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
     *reinterpret_cast<float2*>(dst + 64) = make_float2(m, l);
   };
 
-  // Merged rows of one item: source `it`, row r -> float pointer (O[64], m, l).
-  // Cluster: recv[it][k] (in the ring) with r = c + k * nitems.  Global:
-  // part[b][h][it][r].
-  const size_t bh = static_cast<size_t>(b) * a.Hkv + h;
-  float* part_bh = a.part + bh * a.max_items * rows_alloc * kAttnRow;
+  // ---- items -> owners: CTA c of the cluster owns rows c, c + nitems, ...
+  // Outgoing rows [owner][slot][kAttnRow] over Q and P, received rows
+  // recv[it][k] (row c + k * nitems of item `it`) in the rings.
+  float* stage = reinterpret_cast<float*>(sQ);
   float* recv = reinterpret_cast<float*>(ring);
-  const int rpo = (rows_alloc + nitems - 1) / nitems;   // cluster: rows per owner
-  bool got = true;
-  int my_rows;
-  if (in_cluster) {
-    // ---- items -> owners.  stage [owner][slot][kAttnRow] over Q and P.
-    float* stage = reinterpret_cast<float*>(sQ);
-    const int blk_floats = rpo * kAttnRow;
-    if (row_thread)
-      put_row(stage + static_cast<size_t>(r % nitems) * blk_floats + (r / nitems) * kAttnRow);
-    fence_proxy_async_smem();
-    __syncthreads();
-    free_tmem();
-    cluster_arrive_release();
-    cluster_wait();   // every CTA of the cluster is done with its pages: receive buffers idle
-    if (threadIdx.x == 0) {
-      const uint32_t bytes = static_cast<uint32_t>(blk_floats * 4);
-      const uint32_t dst_local = smem_u32(recv) + static_cast<uint32_t>(c) * bytes;
+  const int rpo = (rows_alloc + nitems - 1) / nitems;   // rows per owner
+  const int blk_floats = rpo * kAttnRow;
+  if (row_thread)
+    put_row(stage + static_cast<size_t>(r % nitems) * blk_floats + (r / nitems) * kAttnRow);
+  fence_proxy_async_smem();
+  __syncthreads();
+  free_tmem();
+  cluster_arrive_release();
+  cluster_wait();   // every CTA of the cluster is done with its pages: receive buffers idle
+  if (threadIdx.x == 0) {
+    const uint32_t bytes = static_cast<uint32_t>(blk_floats * 4);
+    const uint32_t dst_local = smem_u32(recv) + static_cast<uint32_t>(c) * bytes;
 #pragma unroll 1
-      for (int q = 0; q < nitems; ++q)
-        bulk_copy_to_peer(cluster_map(dst_local, static_cast<uint32_t>(q)),
-                          smem_u32(stage) + static_cast<uint32_t>(q) * bytes, bytes,
-                          cluster_map(smem_u32(recv_bar), static_cast<uint32_t>(q)));
-      bulk_commit();
-    }
-    got = mbar_wait(smem_u32(recv_bar), 0, a.err);
-    my_rows = (R - c + nitems - 1) / nitems;
-  } else {
-    // ---- item rows -> global scratch; the last item to arrive merges
-    if (row_thread) put_row(part_bh + (static_cast<size_t>(c) * rows_alloc + r) * kAttnRow);
-    __syncthreads();
-    free_tmem();
-    if (threadIdx.x == 0) {
-      __threadfence();   // behind the barrier: covers the rows every thread wrote
-      s_int[1] = (atomicAdd(a.ticket + bh, 1) == nitems - 1) ? 1 : 0;
-    }
-    __syncthreads();
-    if (!s_int[1]) return;
-    __threadfence();
-    if (threadIdx.x == 0) a.ticket[bh] = 0;   // every item of this launch has arrived
-    my_rows = R;
+    for (int q = 0; q < nitems; ++q)
+      bulk_copy_to_peer(cluster_map(dst_local, static_cast<uint32_t>(q)),
+                        smem_u32(stage) + static_cast<uint32_t>(q) * bytes, bytes,
+                        cluster_map(smem_u32(recv_bar), static_cast<uint32_t>(q)));
+    bulk_commit();
   }
-  auto row_of = [&](int k) { return in_cluster ? c + k * nitems : k; };
-  // source rows: the owner's receive buffer (shared) or the global scratch
-  // (written by other SMs in this launch: read at L2, never from L1)
-  auto src_of = [&](int it, int k) -> const float* {
-    return in_cluster ? recv + (static_cast<size_t>(it) * rpo + k) * kAttnRow
-                      : part_bh + (static_cast<size_t>(it) * rows_alloc + k) * kAttnRow;
-  };
-  auto ld2 = [&](const float* p) {
-    return in_cluster ? *reinterpret_cast<const float2*>(p) : __ldcg(reinterpret_cast<const float2*>(p));
-  };
-  auto ld4 = [&](const float* p) {
-    return in_cluster ? *reinterpret_cast<const float4*>(p) : __ldcg(reinterpret_cast<const float4*>(p));
-  };
+  const bool got = mbar_wait(smem_u32(recv_bar), 0, a.err);
+  const int my_rows = (R - c + nitems - 1) / nitems;
 
-  // ---- merge of items 0..nitems-1 in order for rows row_of(k), k < my_rows.
-  //      mb/lb [item][k] hold m and l, then mb the coefficients w_it / L (one
-  //      thread per row); then one thread per (row, 4 dims) sums coef * O_it.
-  if (in_cluster && threadIdx.x == 0) bulk_wait_read_all();   // outgoing rows have left
-  __syncthreads();
-  // cluster: the received rows fill the ring, the tables go over Q and P (the
-  // outgoing copies have read them); global: the tables go in the ring
-  float* mb = reinterpret_cast<float*>(in_cluster ? sQ : ring);
-  float* lb = mb + static_cast<size_t>(nitems) * rows_alloc;
-  const bool fits = 2 * nitems * rows_alloc * 4 <= (in_cluster ? kAttnRingOff : kAttnRingBytes);
-  if (!fits && threadIdx.x == 0) atomicExch(a.err, kErrBounds);
-  if (fits) {
+  // ---- merge of items 0..nitems-1 in order for the owned rows: one thread per
+  //      (row, 4 dims); M = max m_i, w_i = 2^(m_i - M), L = sum w_i l_i,
+  //      O = sum (w_i / L) O_i
 #pragma unroll 1
-    for (int idx = threadIdx.x; idx < nitems * my_rows; idx += blockDim.x) {
-      const int it = idx / my_rows, k = idx - it * my_rows;
-      const float2 ml = ld2(src_of(it, k) + 64);
-      mb[it * rows_alloc + k] = ml.x;
-      lb[it * rows_alloc + k] = ml.y;
+  for (int idx = threadIdx.x; idx < my_rows * 16; idx += blockDim.x) {
+    const int k = idx >> 4, d4 = (idx & 15) * 4;
+    const float* row = recv + static_cast<size_t>(k) * kAttnRow;
+    float M = -INFINITY, L = 0.f;
+#pragma unroll 4
+    for (int it = 0; it < nitems; ++it) M = fmaxf(M, row[it * blk_floats + 64]);
+#pragma unroll 4
+    for (int it = 0; it < nitems; ++it) {
+      const float2 ml = *reinterpret_cast<const float2*>(row + it * blk_floats + 64);
+      L += (ml.x == -INFINITY ? 0.f : exp2f(ml.x - M)) * ml.y;
+    }
+    const float inv = 1.0f / L;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+    for (int it = 0; it < nitems; ++it) {
+      const float mi = row[it * blk_floats + 64];
+      const float4 v = *reinterpret_cast<const float4*>(row + it * blk_floats + d4);
+      const float w = (mi == -INFINITY ? 0.f : exp2f(mi - M)) * inv;
+      acc.x += w * v.x;
+      acc.y += w * v.y;
+      acc.z += w * v.z;
+      acc.w += w * v.w;
+    }
+    if (all_ok && got) {
+      const int rr = c + k * nitems;
+      const int tt = rr * a.g_magic >> 16;
+      const int hq = h * a.G + rr - tt * a.G;
+      __half* dst = a.out + (static_cast<size_t>(tok0 + tt) * a.Hq + hq) * 64 + d4;
+      *reinterpret_cast<__half2*>(dst) = __floats2half2_rn(acc.x, acc.y);
+      *reinterpret_cast<__half2*>(dst + 2) = __floats2half2_rn(acc.z, acc.w);
     }
   }
-  __syncthreads();
-  if (fits) {
-#pragma unroll 1
-    for (int k = threadIdx.x; k < my_rows; k += blockDim.x) {
-      float M = -INFINITY;
-      for (int it = 0; it < nitems; ++it) M = fmaxf(M, mb[it * rows_alloc + k]);
-      float L = 0.f;
-#pragma unroll 1
-      for (int it = 0; it < nitems; ++it) {
-        const float mi = mb[it * rows_alloc + k];
-        const float w = (mi == -INFINITY) ? 0.f : exp2f(mi - M);
-        mb[it * rows_alloc + k] = w;
-        L += w * lb[it * rows_alloc + k];
-      }
-      const float inv = 1.0f / L;
-#pragma unroll 1
-      for (int it = 0; it < nitems; ++it) mb[it * rows_alloc + k] *= inv;
-    }
-  }
-  __syncthreads();
-  if (fits) {
-#pragma unroll 1
-    for (int idx = threadIdx.x; idx < my_rows * 16; idx += blockDim.x) {
-      const int k = idx >> 4, d4 = (idx & 15) * 4;
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 1
-      for (int it0 = 0; it0 < nitems; it0 += 8) {   // 8 loads in flight, summed in order
-        const int n8 = min(8, nitems - it0);
-        float4 v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-          if (u < n8) v[u] = ld4(src_of(it0 + u, k) + d4);
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-          if (u < n8) {
-            const float w = mb[(it0 + u) * rows_alloc + k];
-            acc.x += w * v[u].x;
-            acc.y += w * v[u].y;
-            acc.z += w * v[u].z;
-            acc.w += w * v[u].w;
-          }
-      }
-      if (all_ok && got) {
-        const int rr = row_of(k);
-        const int tt = rr * a.g_magic >> 16;
-        const int t = tok0 + tt;
-        const int hq = h * a.G + rr - tt * a.G;
-        __half* dst = a.out + (static_cast<size_t>(t) * a.Hq + hq) * 64 + d4;
-        *reinterpret_cast<__half2*>(dst) = __floats2half2_rn(acc.x, acc.y);
-        *reinterpret_cast<__half2*>(dst + 2) = __floats2half2_rn(acc.z, acc.w);
-      }
-    }
-  }
+  if (threadIdx.x == 0) bulk_wait_read_all();   // our outgoing rows have left
 }
 
 }  // namespace gs

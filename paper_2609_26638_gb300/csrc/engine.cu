@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "attention.cuh"
+#include "attention_stream.cuh"
 #include "denoise.cuh"
 #include "gemm_tc.cuh"
 #include "internal.h"
@@ -125,6 +126,9 @@ cudaError_t gs::ensure_kernel_attributes() {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(attn_paged_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              attn_max_smem_bytes());
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(attn_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kAttnStreamSmem);
   if (e == cudaSuccess)   // clusters of up to 16 attention items
     e = cudaFuncSetAttribute(attn_paged_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e == cudaSuccess && dev < 64) done |= 1ull << dev;
@@ -140,6 +144,9 @@ bool attn_use_cluster(int items, int blocks_x_heads) {
 cudaError_t launch_attention(const CUtensorMap& tm, const AttnArgs& a, int n_blocks,
                              cudaStream_t s, bool pdl) {
   dim3 grid(a.max_items, a.Hkv, n_blocks);
+  if (!a.cluster)
+    return launch_ex(attn_stream_kernel, dim3(a.Hkv, n_blocks, a.max_items), dim3(kAttnThreads), kAttnStreamSmem, s, pdl,
+                     dim3(1, 1, 1), tm, a);
   return launch_ex(attn_paged_kernel, grid, dim3(kAttnThreads), kAttnSmemBytes, s, pdl,
                    dim3(a.cluster ? a.max_items : 1, 1, 1), tm, a);
 }
@@ -566,6 +573,7 @@ int run_attention(gs_handle* h, int layer, int T, const AttnLaunch& L) {
   a.split_pages = L.split_pages;
   a.max_items = L.max_items;
   a.cluster = attn_use_cluster(L.max_items, L.n_seq * g.n_sub * c.n_kv_heads) ? 1 : 0;
+  a.early = 1;
   a.part = h->attn_part;
   a.ticket = h->attn_ticket;
   a.err = h->err_word;
@@ -1555,9 +1563,14 @@ size_t gs_attention_scratch_bytes(int n_seq, int W, int n_heads, int n_kv_heads,
 }  // extern "C"
 
 namespace {
+// Also zeroes the error word and the merge tickets (the kernel leaves the
+// tickets at zero, but the scratch may hold anything).
 __global__ void attn_standalone_prep(int mode, const int32_t* n, int n_seq, int W, int32_t* lim,
-                                     int32_t* blk_slot) {
+                                     int32_t* blk_slot, int* ticket, int n_tickets, int* err) {
+  pdl_trigger();
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx == 0) *err = 0;
+  if (idx < n_tickets) ticket[idx] = 0;
   if (idx >= n_seq * W) return;
   const int b = idx / W, i = idx % W;
   const int ns = n[b];
@@ -1599,10 +1612,10 @@ int gs_attention(int mode, const void* q, const void* kv, int n_pages, const int
   const uint64_t rows = static_cast<uint64_t>(n_pages) * 2 * n_kv_heads * 64;
   if (rows >= (1ull << 31) || !make_map(&tm, kv, rows, 64, 64)) return GS_ERR_INVALID_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // the merge tickets start at zero (the kernel leaves them at zero)
-  if (cudaMemsetAsync(ticket, 0, blocks * n_kv_heads * sizeof(int), s) != cudaSuccess)
-    return GS_ERR_CUDA;
-  attn_standalone_prep<<<cdiv(n_seq * W, 128), 128, 0, s>>>(mode, n, n_seq, W, lim, blk_slot);
+  const int n_tickets = static_cast<int>(blocks) * n_kv_heads;
+  attn_standalone_prep<<<cdiv(std::max(n_seq * W, n_tickets), 128), 128, 0, s>>>(
+      mode, n, n_seq, W, lim, blk_slot, ticket, n_tickets, err);
+  if (cudaGetLastError() != cudaSuccess) return GS_ERR_CUDA;
   AttnArgs a;
   a.q = static_cast<const __half*>(q);
   a.lim = lim;
@@ -1628,8 +1641,9 @@ int gs_attention(int mode, const void* q, const void* kv, int n_pages, const int
   a.part = part;
   a.ticket = ticket;
   a.err = err;
-  return launch_attention(tm, a, static_cast<int>(blocks), s, false) == cudaSuccess ? GS_OK
-                                                                                   : GS_ERR_CUDA;
+  a.early = 0;   // the launch before this one writes the limits
+  return launch_attention(tm, a, static_cast<int>(blocks), s, true) == cudaSuccess ? GS_OK
+                                                                                  : GS_ERR_CUDA;
 }
 
 size_t gs_linear_scratch_bytes(int M, int N, int split_k) {

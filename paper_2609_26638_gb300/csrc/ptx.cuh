@@ -55,24 +55,28 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
-// The retries of mbar_wait, bounded by limit_ns of %globaltimer.  Out of line:
-// every wait of a kernel shares this copy, so a pipeline's instructions stay in
-// the instruction cache (a kernel here runs for a few microseconds; one line
-// fetched from beyond the SM's cache costs a tenth of one, or more under load).
-static __device__ __noinline__ bool mbar_wait_retry(uint32_t bar, uint32_t parity, int* err,
-                                                    uint64_t limit_ns) {
-#pragma unroll 1
-  for (int i = 0; i < 256; ++i)
-    if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = global_timer_ns();
-  while (true) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if (global_timer_ns() - t0 > limit_ns) {
-      atomicExch(err, kErrTimeout);
-      return false;
-    }
-    __nanosleep(128);
-  }
+// The retries of mbar_wait, bounded by limit_ns of %globaltimer: a dozen
+// instructions in place, so a pipeline's code stays in the instruction cache
+// (retries unrolled in C took 0.7 KB per wait; shared out of line, the call made
+// values that live across a wait spill).  try_wait suspends, so the loop is slow.
+__device__ __forceinline__ bool mbar_wait_retry(uint32_t bar, uint32_t parity, uint64_t limit_ns) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t.reg .u64 t0, t1;\n\t"
+      "mov.u64 t0, %%globaltimer;\n"
+      "retry_%=:\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "@p bra done_%=;\n\t"
+      "mov.u64 t1, %%globaltimer;\n\t"
+      "sub.u64 t1, t1, t0;\n\t"
+      "setp.gt.u64 q, t1, %3;\n\t"
+      "@!q bra retry_%=;\n"
+      "done_%=:\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity), "l"(limit_ns)
+      : "memory");
+  return ok != 0;
 }
 
 // Wait for the phase with the given parity; false (and the error word set)
@@ -84,7 +88,9 @@ static __device__ __noinline__ bool mbar_wait_retry(uint32_t bar, uint32_t parit
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* err,
                                           uint64_t limit_ns = kWaitLimitNs) {
   if (mbar_try_wait(bar, parity)) return true;
-  return mbar_wait_retry(bar, parity, err, limit_ns);
+  if (mbar_wait_retry(bar, parity, limit_ns)) return true;
+  atomicExch(err, kErrTimeout);
+  return false;
 }
 
 // Position in a ring of `n` stages: the stage and the parity of its use,

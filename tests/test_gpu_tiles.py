@@ -1,13 +1,18 @@
-"""GPU parity at the edges of the persistent GEMM's tiles: token tiles of 32 to 256
-rows and their remainders, odd k-block counts, in-CTA K chunks, the resident
-token tile, SwiGLU gates outside the fast quotient's range.
+"""GPU parity at the edges of the persistent GEMM's and the streaming attention's
+tiles: token tiles of 32 to 256 rows and their remainders, odd k-block counts,
+in-CTA K chunks, the resident token tile, SwiGLU gates outside the fast
+quotient's range; attention launches of more than one wave with one item, more
+than eight items, windows of one row and sub-blocks of two rows.
 
 References and tolerances as in test_gpu_kernels.py (fp32 matmul of the same
-fp16 operands, 2^-11 relative for fp16 stores)."""
+fp16 operands, 2^-11 relative for fp16 stores; the oracle's float64 softmax)."""
+import numpy as np
 import pytest
 import torch
 
-from tests.test_gpu_kernels import DEV, _linear
+import synth
+from oracle import decode as od
+from tests.test_gpu_kernels import DEV, _linear, _oracle_attn, _paged, _run_attention
 
 pytestmark = pytest.mark.gpu
 
@@ -72,3 +77,25 @@ def test_swiglu_gates_of_any_size(gs, M, split):
     _linear(gs, x, w, M, F, K, gs.EPI_SWIGLU, split, y)
     torch.testing.assert_close(y.double(), ref, rtol=2e-3, atol=1e-3)
     assert float(y[M // 2].abs().max()) == 0.0
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("B,W,lo,hi,Hq,Hkv,sp", [
+    (40, 1, 1, 200, 16, 8, 4),       # rows of one token: two per block
+    (24, 17, 30, 900, 16, 8, 1),     # up to fifteen items, merged through scratch
+    (6, 65, 500, 1400, 16, 8, 3),    # sub-blocks of 128 and of 2 rows
+    (80, 9, 0, 60, 4, 4, 2),         # one item per sequence
+])
+def test_attention_streams_items(gs, mode, B, W, lo, hi, Hq, Hkv, sp):
+    rng = np.random.default_rng(B + W + mode)
+    ns = [int(v) for v in rng.integers(lo, hi + 1, B)]
+    q, k, v = synth.attn_inputs(B, W, hi + W + 1, Hq, Hkv, index=B + mode)
+    pool, pt, _ = _paged(k, v, rng)
+    got = _run_attention(gs, mode, q, pool, pt, np.array(ns), W, Hq, Hkv, sp)
+    K = W - 1
+    for b in sorted({0, B - 1, int(np.argmax(ns)), int(np.argmin(ns))}):
+        allowed = od.draft_allowed(ns[b], K) if mode == 0 else od.verify_allowed(ns[b], K)
+        nk = allowed.shape[1]
+        want = _oracle_attn(q[b].astype(np.float64), k[b, :nk].astype(np.float64),
+                            v[b, :nk].astype(np.float64), allowed, Hq, Hkv)
+        np.testing.assert_allclose(got[b], want, rtol=5e-3, atol=5e-3)
