@@ -1711,8 +1711,14 @@ int gs_linear(const void* x, const void* w, void* y, int M, int N, int K, int ep
   a.logits = nullptr;
   a.w_scale = 1.f;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (clear_words(static_cast<int*>(scratch), head_bytes / 4, s) != cudaSuccess) return GS_ERR_CUDA;
-  return launch_gemm(bn, epilogue, tw, tx, a, feat_tiles, tok_tiles, s, true) == cudaSuccess
+  // A split launch (up to 64 rows) is shorter than the host's two calls, and a
+  // memset is the cheaper of them there (9.3 us a call against 10.2 at 17 x 2048 x
+  // 1024); longer launches gain from overlapping their prologue.
+  const bool overlap = p.splits == 1;
+  if ((overlap ? clear_words(static_cast<int*>(scratch), head_bytes / 4, s)
+               : cudaMemsetAsync(scratch, 0, head_bytes, s)) != cudaSuccess)
+    return GS_ERR_CUDA;
+  return launch_gemm(bn, epilogue, tw, tx, a, feat_tiles, tok_tiles, s, overlap) == cudaSuccess
              ? GS_OK
              : GS_ERR_CUDA;
 }

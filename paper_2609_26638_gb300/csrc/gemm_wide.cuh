@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(WideShape<BN>::kThreads, 1)
 #pragma unroll
           for (int q = 0; q < 16; ++q) ss += part[q];
           for (int q = 16; q < a.n_ssp; ++q) ss += sp[q];
-          rs_s[t] = rsqrtf(ss * a.inv_d + a.eps);
+          rs_s[t] = rsqrtf(ss * a.inv_d + a.eps) * a.w_scale;
         }
       }
       // the chunks: running sum in registers, its total over the last buffer

@@ -75,9 +75,9 @@ inline int wide_index(int bn) {
 }
 
 // The token tile with the least estimated time: rounds of tiles over the SMs,
-// each the longer of its k-blocks and its epilogue slices (about 700 cycles per
-// 32 tokens of a group; one group of warps at 32 rows, else two), and the last
-// tile's epilogue, which nothing overlaps.  The wider on a tie.
+// each the longer of its k-blocks and its epilogue slices (about 2,000 cycles
+// per 32 tokens of a group; one group of warps at 32 rows, else two), and the
+// last tile's epilogue, which nothing overlaps.  The wider on a tie.
 inline int wide_bn(int feat_tiles, int T, int nkb) {
   int best = 32;
   long long best_cost = -1;
@@ -86,7 +86,7 @@ inline int wide_bn(int feat_tiles, int T, int nkb) {
     const long long tiles = static_cast<long long>(feat_tiles) * ((T + bn - 1) / bn);
     const long long rounds = (tiles + kNumSMs - 1) / kNumSMs;
     const long long main = static_cast<long long>(nkb) * kWideCycles[i];
-    const long long epi = 700ll * ((bn / (bn >= 64 ? 2 : 1) + 31) / 32);
+    const long long epi = 2000ll * ((bn / (bn >= 64 ? 2 : 1) + 31) / 32);
     const long long cost = rounds * (main > epi ? main : epi) + epi;
     if (best_cost < 0 || cost < best_cost) {
       best_cost = cost;
