@@ -1648,15 +1648,15 @@ int gs_attention(int mode, const void* q, const void* kv, int n_pages, const int
 
 size_t gs_linear_scratch_bytes(int M, int N, int split_k) {
   if (M < 1 || N < 64 || split_k < 1) return 0;
-  // the larger of the plans for an N-row and a 2N-row (SwiGLU) weight; only a
-  // launch that splits K across CTAs needs counters (and partials, unless its
-  // CTAs form clusters), and its tiles do not depend on K
+  // the larger of the plans for an N-row and a 2N-row (SwiGLU) weight: counters for
+  // windows of up to 64 rows, whatever the split, and partials for splits that form
+  // no cluster; launches over 64 rows never split K across CTAs and use neither
   size_t counters = 0, partial = 0;
   for (int w_rows : {N, 2 * N}) {
     const GemmPlan p = plan_split(w_rows, M, split_k, split_k);
-    if (p.splits == 1) continue;
+    if (p.splits == 1 && M > 64) continue;
     counters = std::max(counters, static_cast<size_t>(p.tok_tiles) * p.feat_tiles);
-    if (!gemm_cluster_ok(p.bn, p.splits))
+    if (p.splits > 1 && !gemm_cluster_ok(p.bn, p.splits))
       partial = std::max(partial, static_cast<size_t>(p.splits) * p.tok_tiles * p.feat_tiles *
                                       p.bn * 128);
   }
