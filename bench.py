@@ -71,10 +71,10 @@ _CSRC = os.path.join(ROOT, "paper_2609_26638_gb300", "csrc")
 NCU_TRAFFIC = {
     "attention_b1": dict(sources=("attention.cuh", "ptx.cuh"), bytes=4990976, algorithmic=4823040,
                          sha256="c4154e97724194c54884ba6a96d4f34400276927858e81f4dd4810b09e00183e"),
-    "attention_serve": dict(sources=("attention.cuh", "ptx.cuh"), bytes=233378304,
+    "attention_serve": dict(sources=("attention.cuh", "attention_stream.cuh", "ptx.cuh"), bytes=233378304,
                             algorithmic=225173504,
                             sha256="f2eb4e50dce5541dd1624732eca164b8f2d58dde484e3e6a86061e1e6dbac85a"),
-    "lm_head_b1": dict(sources=("gemm_tc.cuh", "gemm.cu", "ptx.cuh"), bytes=124897280,
+    "lm_head_b1": dict(sources=("gemm_tc.cuh", "gemm_wide.cuh", "gemm_wide.cu", "ptx.cuh"), bytes=124897280,
                        algorithmic=121669768,
                        sha256="cf843ef01b07ec00b2c8f45ea0314bd187665ee6d84ddb19be137f33e3a34ecb"),
 }
@@ -444,7 +444,7 @@ def kernel_table(eng, cfg, slots, K, B, R, force, out_tok, out_cnt, out_done, re
     timing = ("CUDA event nodes after every launch of one forced decode, each round captured and "
               "replayed as a graph (no host gaps; no launch overlap across an event)")
     if dk["bound"] == "tensor":
-        roof = {"kernel": f"{dom} (gemm_tc_kernel), {T} rows", "bound": "tensor",
+        roof = {"kernel": f"{dom} (gemm_tc_kernel / gemm_wide_kernel), {T} rows", "bound": "tensor",
                 "achieved": dk["tflop_s"], "peak": bf16_tf, "unit": "TFLOP/s",
                 "frac": dk["frac_tensor"], "peak_source": src + " bf16 burst (fp16 runs at the same rate)",
                 "algorithmic_flops_per_launch": dk["flops_per_launch"],
@@ -455,7 +455,7 @@ def kernel_table(eng, cfg, slots, K, B, R, force, out_tok, out_cnt, out_done, re
         if dom == "attention":
             traffic = ncu_traffic("attention_b1" if B == 1 else "attention_serve",
                                   dk["bytes_per_launch"])
-        roof = {"kernel": f"{dom} (gemm_tc_kernel / attn_paged_kernel by kind), {T} rows",
+        roof = {"kernel": f"{dom} (gemm_*_kernel / attn_*_kernel by kind), {T} rows",
                 "bound": "hbm", "achieved": dk["gb_s"], "peak": hbm, "unit": "GB/s",
                 "frac": dk["frac_hbm"], "peak_source": src,
                 "algorithmic_bytes_per_launch": dk["bytes_per_launch"],
@@ -537,7 +537,7 @@ def lm_head_roofline(cfg, K, dev):
     t = _time_kernel(fn, 30)
     algo = N * Kd * 2 + M * Kd * 2 + M * 8
     achieved = algo / t / 1e9
-    return {"kernel": "gemm_tc_kernel<32, argmax> (LM head 17x59392x1024)", "bound": "hbm",
+    return {"kernel": "gemm_wide_kernel<32, argmax> (LM head 17x59392x1024)", "bound": "hbm",
             "achieved": round(achieved, 1), "peak": hbm, "unit": "GB/s",
             "frac": round(achieved / hbm, 4), "peak_source": src, "algorithmic_bytes": algo,
             "us_per_launch": round(t * 1e6, 2), "traffic": ncu_traffic("lm_head_b1", algo)}
@@ -577,7 +577,7 @@ def gemm_serve_rooflines(cfg, dev, T=544):
         t = _time_kernel(fn, 20)
         flops = 2 * T * wrows * Kd
         tf = flops / t / 1e12
-        out.append({"kernel": f"gemm_tc_kernel ({name}, {T} x {wrows} x {Kd}, split-K {split})",
+        out.append({"kernel": f"gemm_wide_kernel ({name}, {T} x {wrows} x {Kd}, split-K {split})",
                     "bound": "tensor", "achieved": round(tf, 1), "peak": bf16_tf, "unit": "TFLOP/s",
                     "frac": round(tf / bf16_tf, 4), "peak_source": src + " bf16 burst",
                     "flops": flops, "us_per_launch": round(t * 1e6, 2)})
@@ -636,7 +636,7 @@ def attention_roofline(cfg, dev, ns=None, K=16, mode=0):
     keys = int(sum(int(n) + W + mode for n in ns))   # the verify window reaches one slot further
     algo = keys * Hkv * 64 * 2 * 2 + 2 * B * W * Hq * 64 * 2
     achieved = algo / t / 1e9
-    return {"kernel": f"attn_paged_kernel ({'verify' if mode else 'draft'}, {B} seqs, mean cached "
+    return {"kernel": f"attention ({'verify' if mode else 'draft'}, {B} seqs, mean cached "
                       f"{int(ns.mean())}, K={K}, {sp} pages per item)", "bound": "hbm",
             "achieved": round(achieved, 1), "peak": hbm, "unit": "GB/s",
             "frac": round(achieved / hbm, 4), "kv_bytes": algo, "us_per_launch": round(t * 1e6, 2),

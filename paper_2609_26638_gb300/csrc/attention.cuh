@@ -215,6 +215,12 @@ __device__ __forceinline__ void attn_store_q(uint8_t* sQ, int R, const uint4 (&v
   }
 }
 
+// Where the softmax warps' rings stand, kept from one item to the next.
+struct AttnRings {
+  RingPos s;   // S / P buffer of the next page
+  RingPos v;   // V^T ring stage of the next page
+};
+
 // Online softmax over the item's pages for one warp and the rows of its lane
 // quarter.  S comes from TMEM in the 16x256b layout, so a row is spread over
 // four neighbouring threads and a set of 8 rows costs a thread 16 columns,
@@ -234,11 +240,6 @@ __device__ __forceinline__ void attn_store_q(uint8_t* sQ, int R, const uint4 (&v
 // unrolled variants this replaces spent 10 k of a CTA's 34 k cycles on that.
 // Waits are bounded; a warp whose wait ran out keeps arriving on the MMA
 // warp's barriers to the last page.  Returns false if a wait ran out.
-struct AttnRings {
-  RingPos s;   // S / P buffer of the next page
-  RingPos v;   // V^T ring stage of the next page
-};
-
 __device__ __forceinline__ bool attn_softmax(const AttnArgs& a, const AttnSync& y, uint32_t tmem,
                                              int warp, int nset, int np, int p_begin,
                                              const int (&lim)[4], AttnRings& rg) {
