@@ -69,14 +69,14 @@ def schedule_rounds(sched: np.ndarray, max_new: int) -> int:
 # traffic grows with the keys read: K and V rows, once each).
 _CSRC = os.path.join(ROOT, "paper_2609_26638_gb300", "csrc")
 NCU_TRAFFIC = {
-    "attention_b1": dict(sources=("attention.cuh", "ptx.cuh"), bytes=4990976, algorithmic=4823040,
-                         sha256="c4154e97724194c54884ba6a96d4f34400276927858e81f4dd4810b09e00183e"),
-    "attention_serve": dict(sources=("attention.cuh", "attention_stream.cuh", "ptx.cuh"), bytes=233378304,
-                            algorithmic=225173504,
-                            sha256="f2eb4e50dce5541dd1624732eca164b8f2d58dde484e3e6a86061e1e6dbac85a"),
-    "lm_head_b1": dict(sources=("gemm_tc.cuh", "gemm_wide.cuh", "gemm_wide.cu", "ptx.cuh"), bytes=124897280,
-                       algorithmic=121669768,
-                       sha256="cf843ef01b07ec00b2c8f45ea0314bd187665ee6d84ddb19be137f33e3a34ecb"),
+    "attention_b1": dict(sources=("attention.cuh", "ptx.cuh"), bytes=4934144, algorithmic=4823040,
+                         sha256="a3a681e67936a67131bf0807979510cab74ae62f207601b15016df7419539d75"),
+    "attention_serve": dict(sources=("attention.cuh", "attention_stream.cuh", "ptx.cuh"),
+                            bytes=233422592, algorithmic=225173504,
+                            sha256="ba0eda31823029a4f665c31dcefd451641439a391145d9c15ef25ef69d703305"),
+    "lm_head_b1": dict(sources=("gemm_tc.cuh", "gemm_wide.cuh", "gemm_wide.cu", "ptx.cuh"),
+                       bytes=124454144, algorithmic=121669768,
+                       sha256="710e19ffeb4dd8225c89174271693bcf7551391a3e415aaf774c1f7470252928"),
 }
 
 

@@ -179,7 +179,7 @@ int decode_splits(int weight_rows, int K) {
 // (each chunk summed from zero in a TMEM buffer, the chunks added in order), as
 // does every launch that is not split.  The sums and their order are the same.
 // Measured at 544 rows: down projection 22.5 us in clusters of 8 with 64-token
-// tiles, see the persistent kernel's header for its side.
+// tiles against 16.4 in the persistent kernel.
 GemmPlan plan_split(int weight_rows, int T, int S, int nkb) {
   GemmPlan p;
   p.feat_tiles = weight_rows / 128;
