@@ -76,7 +76,7 @@ NCU_TRAFFIC = {
                             sha256="ba0eda31823029a4f665c31dcefd451641439a391145d9c15ef25ef69d703305"),
     "lm_head_b1": dict(sources=("gemm_tc.cuh", "gemm_wide.cuh", "gemm_wide.cu", "ptx.cuh"),
                        bytes=124454144, algorithmic=121669768,
-                       sha256="710e19ffeb4dd8225c89174271693bcf7551391a3e415aaf774c1f7470252928"),
+                       sha256="239775d170ba9d4ae12d02bf55c93c86d37f5d8ac676b82c75a59f28efbb164f"),
 }
 
 
