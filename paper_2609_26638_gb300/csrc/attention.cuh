@@ -498,7 +498,10 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
     for (int i = lane; i < min(np, kAttnPtAhead); i += 32) pt_s[i] = pt[p_begin + i];
     __syncwarp();
     if (elect_one()) {
-      const int safe_pages = a.blk_slot ? a.lim[tok0] / 64 : 0;   // wholly committed pages
+      // pages wholly before the window: the limit of the WINDOW's first token (n or
+      // n + 1); a later sub-block's own limits reach into slots that the kernel
+      // right before this one is still writing
+      const int safe_pages = a.blk_slot ? a.lim[seq * a.QB] / 64 : 0;
       const uint64_t pol = l2_policy_evict_first();
       RingPos rk, rv;
       const uint32_t k_full0 = smem_u32(k_full), k_empty0 = smem_u32(k_empty);

@@ -241,8 +241,10 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
       int lm[4];   // ntok <= 128
 #pragma unroll
       for (int q = 0; q < 4; ++q) lm[q] = lane + 32 * q < ntok ? a.lim[tok0 + lane + 32 * q] : -1;
+      // pages wholly before the window, from the window's first token (a later
+      // sub-block's own limits reach into the window)
+      nsafe = a.blk_slot ? a.lim[seq * a.QB] / 64 : 0;
       const int maxlim = __reduce_max_sync(0xFFFFFFFFu, max(max(lm[0], lm[1]), max(lm[2], lm[3])));
-      nsafe = a.blk_slot ? __shfl_sync(0xFFFFFFFFu, lm[0], 0) / 64 : 0;
       const int npages = maxlim / 64 + 1;
       const int nitems = (npages + a.split_pages - 1) / a.split_pages;
       const bool bad = maxlim < 0 || npages > a.pt_stride || slot < 0 || nitems > a.max_items ||

@@ -255,3 +255,27 @@ def test_round_profile_matches_round(tiny_gain):
 def gs_launches(eng):
     from paper_2609_26638_gb300 import gs
     return gs.gs_round_launches(eng.handle)
+
+
+@pytest.mark.parametrize("K,split_pages,max_ctx", [(16, 0, 512), (31, 0, 512), (31, 1, 2048)])
+def test_windows_of_more_than_128_rows_at_a_page_edge(K, split_pages, max_ctx):
+    """GQA group 8: a window's (K + 1) * 8 rows exceed one query block of 128, and
+    the second block's key limits lie inside the window.  The first window starts
+    a few slots below a page edge, so its own slots complete a page that an item
+    loads first: that page counts as committed for no block of the window.
+    Clusters of items and (32 items of one page) persistent CTAs; in lock-step
+    with the oracle, and as graph launches equal to greedy AR token for token."""
+    cfg = synth.TINY.with_(n_heads=16, n_kv_heads=2)
+    w = synth.make_weights(cfg, seed=9, gain_std=0.1)
+    prompt = synth.make_prompt(cfg, 100, 22, index=K)          # n = 122, edges at 128 and 192
+    eng = new_engine(cfg, w, max_ctx=max_ctx, max_K=K, max_prefill=128, split_pages=split_pages)
+    st, stats = lockstep(eng, Decoder(cfg, w), prompt, K, 48, check_logits=True)
+    print(f"\nK={K}: {stats}")
+    assert st.done and len(st.out) == 48
+    slots = torch.tensor([0], dtype=torch.int32, device=eng.device)
+    outs = []
+    for k in (0, K):
+        x0 = eng.prefill(0, prompt.vis, prompt.text, 80)
+        outs.append([x0] + decode_all(eng, slots, k, 80)[0])
+    assert len(outs[0]) == 80 and outs[1] == outs[0]
+    eng.close()
