@@ -294,7 +294,8 @@ int gs_round_profile(gs_handle *h, const int32_t *slots, int n_seq, int K, const
 int gs_release(gs_handle *h, int slot);
 
 /* Synchronise the stream and report a kernel-side check or bounded-wait
- * failure raised since the last call (then clear it). */
+ * failure raised since the last call (then clear it, and what a launch that gave
+ * up may have left in the workspace's counters). */
 int gs_sync_check(gs_handle *h);
 
 /* Failure-detection self-test (the paper has no counterpart).  Enqueues on

@@ -245,6 +245,7 @@ struct gs_handle {
   float* attn_part = nullptr;
   size_t attn_part_floats = 0;
   int* attn_ticket = nullptr;
+  size_t attn_tickets = 0;
 
   // workspace
   int* err_word = nullptr;
@@ -465,6 +466,7 @@ size_t carve(gs_handle* h, const gs_config& c, void* base) {
     h->attn_part = attn_part;
     h->attn_part_floats = attn_part_floats;
     h->attn_ticket = attn_ticket;
+    h->attn_tickets = attn_blocks * c.n_kv_heads;
     h->err_word = err_word;
     h->wcopy = wcopy;
     h->partial_floats = partial_floats;
@@ -1537,6 +1539,9 @@ int gs_sync_check(gs_handle* h) {
   if (word == 0) return GS_OK;
   const int zero = 0;
   GS_CUDA(h, cudaMemcpy(h->err_word, &zero, 4, cudaMemcpyHostToDevice));
+  // A launch whose wait ran out drops items: the attention's merge tickets, which
+  // every complete launch leaves at zero, may not be.
+  GS_CUDA(h, cudaMemsetAsync(h->attn_ticket, 0, h->attn_tickets * sizeof(int), h->stream));
   if (word == kErrTimeout) return fail(h, GS_ERR_TIMEOUT, "a kernel's bounded wait ran out");
   return fail(h, GS_ERR_DEVICE_CHECK, "a kernel bounds check fired");
 }

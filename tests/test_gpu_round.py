@@ -279,3 +279,62 @@ def test_windows_of_more_than_128_rows_at_a_page_edge(K, split_pages, max_ctx):
         outs.append([x0] + decode_all(eng, slots, k, 80)[0])
     assert len(outs[0]) == 80 and outs[1] == outs[0]
     eng.close()
+
+
+def _merge_tickets(eng):
+    """The attention's merge tickets, one int32 per (query block, KV head): a view
+    into the engine's workspace, found from its end (the pieces behind the tickets,
+    each starting on 256 bytes).  The denoising step counts lie on the way."""
+    c, up = eng.cfg, lambda n: (n + 255) // 256 * 256
+    W, G = c.max_K + 1, c.n_heads // c.n_kv_heads
+    rows = c.max_batch * W
+    weights = sum(t.numel() for lw in eng.layers for n, t in lw.items() if n.startswith("w_"))
+    weights += eng.w["lm_head"].numel()
+    off = eng.ws_bytes
+    for nbytes in (2 * weights, 16 * rows, 4 * rows * c.vocab, 4 * rows * c.vocab,
+                   8 * rows * (c.vocab // 128), 8 * rows * (c.vocab // 128), 256):
+        off -= up(nbytes)
+    words = eng.workspace.view(torch.int32)
+    off -= up(4 * c.max_batch)
+    steps = words[off // 4:off // 4 + c.max_batch]
+    off -= 2 * up(4 * c.max_batch) + up(4 * rows)
+    qb = 128 // G
+    n_sub = -(-W // min(W, qb))
+    T_max = up(max(rows, c.max_prefill, 256))
+    blocks = max(c.max_batch * n_sub, -(-min(c.max_prefill, T_max) // qb))
+    off -= up(4 * blocks * c.n_kv_heads)
+    return words[off // 4:off // 4 + blocks * c.n_kv_heads], steps
+
+
+def test_timeout_report_resets_the_merge_tickets(tiny_gain):
+    """A launch whose wait runs out drops work items, which can leave merge tickets
+    behind; with one left, a later launch would merge before its last item has
+    arrived.  The report of the failure clears them: tickets are planted and the
+    failure raised from the host, and after gs_sync_check the words are zero and a
+    decode through the persistent attention (32 items of one page) commits what it
+    did before."""
+    from paper_2609_26638_gb300 import gs
+    cfg, w, _ = tiny_gain
+    eng = new_engine(cfg, w, max_batch=2, max_ctx=2048, max_K=8, max_prefill=256, split_pages=1)
+    prompt = synth.make_prompt(cfg, 300, 12, index=41)
+    slots = torch.tensor([0], dtype=torch.int32, device=eng.device)
+    tickets, steps = _merge_tickets(eng)
+    out = torch.zeros((3, 8), dtype=torch.int32, device=eng.device)
+    eng.prefill(0, prompt.vis, prompt.text, 40)
+    eng.diffusion_block(slots, 4, 2.0, out[0], out[1], out[2])
+    eng.stream.synchronize()
+    assert steps.tolist() == [4, 0]                      # the view is where it is said to be
+    eng.prefill(0, prompt.vis, prompt.text, 40)
+    before = decode_all(eng, slots, 8, 40)[0]
+    assert not tickets.any()
+    tickets.fill_(1)
+    torch.cuda.synchronize()
+    gs.gs_wait_probe(eng.handle, 1000)
+    with pytest.raises(gs.GsError) as e:
+        eng.check()
+    assert e.value.code == gs.GS_ERR_TIMEOUT
+    torch.cuda.synchronize()
+    assert not tickets.any()
+    eng.prefill(0, prompt.vis, prompt.text, 40)
+    assert decode_all(eng, slots, 8, 40)[0] == before
+    eng.close()
