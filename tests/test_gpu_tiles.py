@@ -6,12 +6,16 @@ than eight items, windows of one row and sub-blocks of two rows.
 
 References and tolerances as in test_gpu_kernels.py (fp32 matmul of the same
 fp16 operands, 2^-11 relative for fp16 stores; the oracle's float64 softmax)."""
+import ctypes
+import subprocess
+
 import numpy as np
 import pytest
 import torch
 
 import synth
 from oracle import decode as od
+from paper_2609_26638_gb300 import build
 from tests.test_gpu_kernels import DEV, _linear, _oracle_attn, _paged, _run_attention
 
 pytestmark = pytest.mark.gpu
@@ -99,3 +103,42 @@ def test_attention_streams_items(gs, mode, B, W, lo, hi, Hq, Hkv, sp):
         want = _oracle_attn(q[b].astype(np.float64), k[b, :nk].astype(np.float64),
                             v[b, :nk].astype(np.float64), allowed, Hq, Hkv)
         np.testing.assert_allclose(got[b], want, rtol=5e-3, atol=5e-3)
+
+
+_SILU_CHECK = r"""
+#include "gemm_tc.cuh"
+__device__ unsigned long long n_bad;
+__device__ unsigned first_bad = 0xFFFFFFFFu;
+// every float bit pattern in [lo, hi]
+__global__ void check(unsigned lo, unsigned hi) {
+  const unsigned long long step = 1ull * gridDim.x * blockDim.x;
+  for (unsigned long long u = lo + 1ull * blockIdx.x * blockDim.x + threadIdx.x; u <= hi; u += step) {
+    const float g = __uint_as_float(static_cast<unsigned>(u));
+    if (__float_as_uint(gs::silu_in_range(g)) != __float_as_uint(gs::silu_any(g))) {
+      atomicAdd(&n_bad, 1ull);
+      atomicMin(&first_bad, static_cast<unsigned>(u));
+    }
+  }
+}
+extern "C" int silu_check(unsigned long long* bad, unsigned* first) {
+  check<<<1216, 256>>>(0u, 0x7149F2CAu);            // +0 .. 1e30
+  check<<<1216, 256>>>(0x80000000u, 0xC2AA0000u);   // -0 .. -85
+  if (cudaDeviceSynchronize() != cudaSuccess) return 1;
+  return cudaMemcpyFromSymbol(bad, n_bad, 8) != cudaSuccess ||
+         cudaMemcpyFromSymbol(first, first_bad, 4) != cudaSuccess;
+}
+"""
+
+
+def test_silu_quotient_equals_the_division_in_every_bit(tmp_path):
+    """silu_in_range against g / (1 + __expf(-g)) for every float of its range,
+    denormals and both zeros included, built with the library's own flags."""
+    assert np.float32(1e30).view(np.uint32) == 0x7149F2CA
+    assert np.float32(-85.0).view(np.uint32) == 0xC2AA0000
+    src, lib = tmp_path / "silu_check.cu", tmp_path / "silu_check.so"
+    src.write_text(_SILU_CHECK)
+    subprocess.run([build._nvcc(), *build.ARCH, *build.FLAGS, "-I", build.CSRC, "-shared", str(src),
+                    "-o", str(lib)], check=True)
+    bad, first = ctypes.c_ulonglong(), ctypes.c_uint()
+    assert ctypes.CDLL(str(lib)).silu_check(ctypes.byref(bad), ctypes.byref(first)) == 0
+    assert bad.value == 0, f"{bad.value} floats differ, the first is 0x{first.value:08X}"
