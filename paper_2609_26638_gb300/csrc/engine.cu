@@ -106,10 +106,6 @@ AttnGeom attn_geom(int W, int G) {
   return {qs, cdiv(W, qs), kAttnMaxRows};
 }
 
-// Items merge inside a cluster when there are at most 16 of them and the
-// launch is about one wave (a cluster waits for free SMs of one GPC, and
-// clusters fragment larger grids); otherwise through global scratch.  Both
-// give the same bits.
 }  // namespace
 
 // Kernel attributes (dynamic shared memory above 48 KB, non-portable cluster
@@ -137,8 +133,16 @@ cudaError_t gs::ensure_kernel_attributes() {
 
 namespace {
 
-bool attn_use_cluster(int items, int blocks_x_heads) {
-  return items <= kAttnMaxCluster && items * blocks_x_heads <= 2 * kNumSMs;
+// Items merge inside a cluster when there are at most 16 of them and the
+// launch is about one wave (a cluster waits for free SMs of one GPC, and
+// clusters fragment larger grids); otherwise through global scratch.  Both
+// give the same bits.  Blocks of more than 96 rows stay in (portable) clusters
+// up to two waves: there a merge of up to 128 rows by one CTA is the longer
+// tail (305-608 CTAs, 100-8000 slots: persistent / cluster time 0.87-1.87, 1.12
+// in the mean; at 66 rows 0.86-1.26, 1.03; above 608 CTAs ragged batches lose).
+bool attn_use_cluster(int items, int blocks_x_heads, int rows) {
+  const int waves = rows > 96 && items <= kMaxClusterSplits ? 2 : 1;
+  return items <= kAttnMaxCluster && items * blocks_x_heads <= waves * 2 * kNumSMs;
 }
 
 cudaError_t launch_attention(const CUtensorMap& tm, const AttnArgs& a, int n_blocks,
@@ -382,7 +386,8 @@ size_t carve(gs_handle* h, const gs_config& c, void* base) {
   const AttnGeom g_dec = attn_geom(W_max, G);
   const int qb_pf = std::max(1, kAttnMaxRows / G);
   const int items_target =
-      attn_use_cluster(kAttnMaxCluster, c.max_batch * g_dec.n_sub * c.n_kv_heads) ? kAttnMaxCluster : 8;
+      attn_use_cluster(kAttnMaxCluster, c.max_batch * g_dec.n_sub * c.n_kv_heads, g_dec.QS * G)
+          ? kAttnMaxCluster : 8;
   int sp = c.split_pages > 0 ? c.split_pages : std::max(2, cdiv(pt_stride, items_target));
   sp = std::max(sp, cdiv(pt_stride, kAttnMaxMergeItems));
   const int items_dec = cdiv(pt_stride, sp);
@@ -574,7 +579,7 @@ int run_attention(gs_handle* h, int layer, int T, const AttnLaunch& L) {
   a.kv_row_base = static_cast<long long>(layer) * h->n_pages * a.rows_per_page;
   a.split_pages = L.split_pages;
   a.max_items = L.max_items;
-  a.cluster = attn_use_cluster(L.max_items, L.n_seq * g.n_sub * c.n_kv_heads) ? 1 : 0;
+  a.cluster = attn_use_cluster(L.max_items, L.n_seq * g.n_sub * c.n_kv_heads, g.QS * h->G) ? 1 : 0;
   a.early = 1;
   a.part = h->attn_part;
   a.ticket = h->attn_ticket;
@@ -1560,7 +1565,8 @@ size_t gs_attention_scratch_bytes(int n_seq, int W, int n_heads, int n_kv_heads,
   cv.take<int32_t>(static_cast<size_t>(n_seq) * W);  // key limits
   cv.take<int32_t>(n_seq);                            // sequence -> page-table row
   cv.take<int>(blocks * n_kv_heads);                  // merge tickets
-  if (!attn_use_cluster(items, static_cast<int>(blocks) * n_kv_heads))   // global merge rows
+  const int rows = g.QS * (n_heads / n_kv_heads);
+  if (!attn_use_cluster(items, static_cast<int>(blocks) * n_kv_heads, rows))   // global merge rows
     cv.take<float>(blocks * n_kv_heads * items * g.rows * kAttnRow);
   return align_up(cv.off, 256);
 }
@@ -1610,7 +1616,8 @@ int gs_attention(int mode, const void* q, const void* kv, int n_pages, const int
   int32_t* lim = cv.take<int32_t>(static_cast<size_t>(n_seq) * W);
   int32_t* blk_slot = cv.take<int32_t>(n_seq);
   int* ticket = cv.take<int>(blocks * n_kv_heads);
-  float* part = attn_use_cluster(items, static_cast<int>(blocks) * n_kv_heads)
+  const bool cluster = attn_use_cluster(items, static_cast<int>(blocks) * n_kv_heads, g.QS * G);
+  float* part = cluster
                     ? nullptr
                     : cv.take<float>(blocks * n_kv_heads * items * g.rows * kAttnRow);
   CUtensorMap tm;
@@ -1642,7 +1649,7 @@ int gs_attention(int mode, const void* q, const void* kv, int n_pages, const int
   a.kv_row_base = 0;
   a.split_pages = split_pages;
   a.max_items = items;
-  a.cluster = attn_use_cluster(items, static_cast<int>(blocks) * n_kv_heads) ? 1 : 0;
+  a.cluster = cluster ? 1 : 0;
   a.part = part;
   a.ticket = ticket;
   a.err = err;

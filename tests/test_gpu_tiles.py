@@ -142,3 +142,27 @@ def test_silu_quotient_equals_the_division_in_every_bit(tmp_path):
     bad, first = ctypes.c_ulonglong(), ctypes.c_uint()
     assert ctypes.CDLL(str(lib)).silu_check(ctypes.byref(bad), ctypes.byref(first)) == 0
     assert bad.value == 0, f"{bad.value} floats differ, the first is 0x{first.value:08X}"
+
+
+@pytest.mark.parametrize("B,W,Hq,Hkv,sp,n", [
+    (4, 65, 16, 8, 2, 700),        # 4 x 2 x 8 x 6 = 384 CTAs in clusters, blocks of 128 and 2 rows
+    (3, 97, 16, 8, 2, 400),        # 4 items: 192 CTAs, one wave
+    (14, 17, 16, 2, 3, 1200),      # 14 x 2 x 2 x 7 = 392 CTAs, blocks of 128 and 8 rows
+])
+def test_attention_clusters_of_two_waves(gs, B, W, Hq, Hkv, sp, n):
+    """Blocks of more than 96 rows in clusters of up to eight items, one to two
+    waves of CTAs: the same rows as each sequence's own launch (one wave), and the
+    oracle's masked softmax."""
+    rng = np.random.default_rng(B)
+    ns = [n - 37 * b for b in range(B)]
+    q, k, v = synth.attn_inputs(B, W, n + W + 1, Hq, Hkv, index=B)
+    pool, pt, _ = _paged(k, v, rng)
+    got = _run_attention(gs, 1, q, pool, pt, np.array(ns), W, Hq, Hkv, sp)
+    for b in (0, B - 1):
+        one = _run_attention(gs, 1, q[b:b + 1], pool, pt[b:b + 1], np.array(ns[b:b + 1]), W, Hq, Hkv, sp)
+        assert np.array_equal(got[b], one[0])
+        allowed = od.verify_allowed(ns[b], W - 1)
+        nk = allowed.shape[1]
+        want = _oracle_attn(q[b].astype(np.float64), k[b, :nk].astype(np.float64),
+                            v[b, :nk].astype(np.float64), allowed, Hq, Hkv)
+        np.testing.assert_allclose(got[b], want, rtol=5e-3, atol=5e-3)
