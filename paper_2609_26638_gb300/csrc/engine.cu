@@ -178,16 +178,24 @@ int decode_splits(int weight_rows, int K) {
 }
 
 // Decode windows of up to 64 tokens split K across the CTAs of a cluster: one
-// or two token tiles of few feature tiles would leave most SMs idle.  Wider
+// or two token tiles of few feature tiles would leave most SMs idle.  Other wider
 // launches reduce the same K chunks inside each CTA of the persistent kernel
 // (each chunk summed from zero in a TMEM buffer, the chunks added in order), as
 // does every launch that is not split.  The sums and their order are the same.
-// Measured at 544 rows: down projection 22.5 us in clusters of 8 with 64-token
-// tiles against 16.4 in the persistent kernel.
+// Above 64 rows the persistent kernel's time is one tile's serial K, whatever the
+// rows: clusters of 8 with 64-token tiles keep the launches whose CTAs all fit
+// (two per SM) and have at least 8 k-blocks each.  us per launch, cluster /
+// persistent, as graph nodes: 1024 x 4096 weight 9.4 / 14.1 at 65 rows, 10.7 /
+// 14.2 at 256 (256 CTAs), 15.0 / 14.3 at 320 (320 CTAs), 20.7 / 14.5 at 544;
+// 2048 x 8192 13.4 / 22.0 at 65, 21.0 / 21.9 at 129; 256 x 4096 7.2 / 13.3 at 65,
+// 9.5 / 14.1 at 544.  Clusters of 4 stay below one wave's worth of gain (4096 x
+// 2048: 11.3 / 9.9 at 128 rows, 4096 x 4096 14.1 / 14.0).
 GemmPlan plan_split(int weight_rows, int T, int S, int nkb) {
   GemmPlan p;
   p.feat_tiles = weight_rows / 128;
-  if (S > 1 && T <= 64) {
+  const bool clusters = S == kMaxClusterSplits && nkb / S >= 8 &&
+                        static_cast<long long>(p.feat_tiles) * cdiv(T, 64) * S <= 2 * kNumSMs;
+  if (S > 1 && (T <= 64 || clusters)) {
     p.splits = S;
     p.chunks = 1;
     p.bn = T <= 32 ? 32 : 64;
@@ -1662,7 +1670,7 @@ size_t gs_linear_scratch_bytes(int M, int N, int split_k) {
   if (M < 1 || N < 64 || split_k < 1) return 0;
   // the larger of the plans for an N-row and a 2N-row (SwiGLU) weight: counters for
   // windows of up to 64 rows, whatever the split, and partials for splits that form
-  // no cluster; launches over 64 rows never split K across CTAs and use neither
+  // no cluster; launches over 64 rows split K inside a CTA or a cluster and use neither
   size_t counters = 0, partial = 0;
   for (int w_rows : {N, 2 * N}) {
     const GemmPlan p = plan_split(w_rows, M, split_k, split_k);
@@ -1692,8 +1700,8 @@ int gs_linear(const void* x, const void* w, void* y, int M, int N, int K, int ep
       (reinterpret_cast<uintptr_t>(y) & 15))
     return GS_ERR_INVALID_ARG;
   if (ensure_kernel_attributes() != cudaSuccess) return GS_ERR_CUDA;
-  // split-K as the decoder plans it: across the CTAs of a cluster or through
-  // global scratch (up to 64 rows), as chunks inside each CTA (wider)
+  // split-K as the decoder plans it: across the CTAs of a cluster, through global
+  // scratch (up to 64 rows), or as chunks inside each CTA
   const int w_rows = epilogue == kEpiSwiGLU ? 2 * N : N;
   const GemmPlan p = plan_split(w_rows, M, split_k, K / 64);
   const int bn = p.bn, tok_tiles = p.tok_tiles, feat_tiles = p.feat_tiles;
@@ -1704,11 +1712,11 @@ int gs_linear(const void* x, const void* w, void* y, int M, int N, int K, int ep
   Carver cv(scratch);
   GemmArgs a = {};
   a.err = cv.take<int>(64);
-  if (p.splits > 1) a.counters = cv.take<int>(static_cast<size_t>(tok_tiles) * feat_tiles);
+  a.cluster = gemm_cluster_ok(bn, p.splits) ? 1 : 0;
+  if (p.splits > 1 && !a.cluster) a.counters = cv.take<int>(static_cast<size_t>(tok_tiles) * feat_tiles);
   // The error word and the per-tile arrival counters of the global split-K
   // path must start at zero, whatever the caller's scratch held before.
   const size_t head_bytes = cv.off;
-  a.cluster = p.splits > 1 && gemm_cluster_ok(bn, p.splits) ? 1 : 0;
   a.partial = p.splits > 1 && !a.cluster
                   ? cv.take<float>(static_cast<size_t>(p.splits) * tok_tiles * feat_tiles * bn * 128)
                   : nullptr;
@@ -1723,10 +1731,10 @@ int gs_linear(const void* x, const void* w, void* y, int M, int N, int K, int ep
   a.logits = nullptr;
   a.w_scale = 1.f;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // A split launch (up to 64 rows) is shorter than the host's two calls, and a
-  // memset is the cheaper of them there (9.3 us a call against 10.2 at 17 x 2048 x
-  // 1024); longer launches gain from overlapping their prologue.
-  const bool overlap = p.splits == 1;
+  // A launch of up to 64 rows that is split is shorter than the host's two calls,
+  // and a memset is the cheaper of them there (9.3 us a call against 10.2 at 17 x
+  // 2048 x 1024); longer launches gain from overlapping their prologue.
+  const bool overlap = p.splits == 1 || M > 64;
   if ((overlap ? clear_words(static_cast<int*>(scratch), head_bytes / 4, s)
                : cudaMemsetAsync(scratch, 0, head_bytes, s)) != cudaSuccess)
     return GS_ERR_CUDA;

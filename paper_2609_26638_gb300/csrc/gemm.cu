@@ -22,15 +22,17 @@ static cudaError_t launch_one(const CUtensorMap& tmW, const CUtensorMap& tmX, Ge
   // Pipeline depth, never more than the k-blocks one CTA loads.  Decode
   // windows (up to 64 rows): a fixed depth that leaves room for a second
   // resident CTA and for the neighbouring kernels' CTAs that overlap it under
-  // programmatic dependent launch.  Wider tiles stream K through each CTA: the
+  // programmatic dependent launch.  Wider launches stream K through each CTA: the
   // deepest pipeline that still fits the CTAs one SM holds (one when the grid
   // is at most one CTA per SM, else two), since bytes in flight per SM set
-  // their load rate.
+  // their load rate.  Clusters always two: with one CTA per SM a cluster of 8
+  // waits for 8 empty SMs of one GPC (1024 x 4096 weight, 68 rows, 128 CTAs:
+  // 17.4 us in the decoder's graph, 13.3 with two).
   const bool cl = a.splits > 1 && a.cluster;
   int want = S::kStagesDefault;
   if (a.M > 64)
-    want = S::stages_fitting(static_cast<long>(feat_tiles) * tok_tiles * a.splits <= kNumSMs ? 1 : 2,
-                             EPI, cl);
+    want = S::stages_fitting(
+        !cl && static_cast<long>(feat_tiles) * tok_tiles * a.splits <= kNumSMs ? 1 : 2, EPI, cl);
   const int kb = a.kb_per_split;
   a.stages = kb < S::kStagesMin ? S::kStagesMin : (kb > want ? want : kb);
   dim3 grid(tok_tiles, feat_tiles, a.splits);

@@ -166,3 +166,30 @@ def test_attention_clusters_of_two_waves(gs, B, W, Hq, Hkv, sp, n):
         want = _oracle_attn(q[b].astype(np.float64), k[b, :nk].astype(np.float64),
                             v[b, :nk].astype(np.float64), allowed, Hq, Hkv)
         np.testing.assert_allclose(got[b], want, rtol=5e-3, atol=5e-3)
+
+
+@pytest.mark.parametrize("N,K,Ms", [(1024, 4096, (65, 128, 129, 256, 257, 320)),
+                                    (2048, 8192, (65, 128, 129)), (256, 4096, (65, 600, 1216, 1217))])
+def test_clusters_above_64_rows(gs, N, K, Ms):
+    """Splits of eight over windows of more than 64 rows, on both sides of the
+    launch size up to which they run as clusters (304 CTAs): the first rows' bits
+    are those of a 17-row window, the result is the fp32 matmul's, and a scratch
+    of the stated size full of stale bytes serves, its error word left at zero."""
+    g = torch.Generator(device=DEV).manual_seed(N + K)
+    x = torch.randn(max(Ms), K, device=DEV, generator=g).half()
+    w = (0.02 * torch.randn(N, K, device=DEV, generator=g)).half()
+    base = torch.randn(max(Ms), N, device=DEV, generator=g)
+    few = base[:17].clone()
+    _linear(gs, x[:17].contiguous(), w, 17, N, K, gs.EPI_RESID_F32, 8, few)
+    for M in Ms:
+        xm = x[:M].contiguous()
+        y = base[:M].clone()
+        sb = gs.gs_linear_scratch_bytes(M, N, 8)
+        scratch = torch.full((sb,), 0x7F, dtype=torch.uint8, device=DEV)
+        gs.gs_linear(xm.data_ptr(), w.data_ptr(), y.data_ptr(), M, N, K, gs.EPI_RESID_F32, 8,
+                     scratch.data_ptr(), sb, torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        assert torch.equal(y[:17], few), M
+        ref = xm.float() @ w.float().T
+        torch.testing.assert_close(y, base[:M] + ref, rtol=1e-4, atol=1e-4 * ref.abs().max().item())
+        assert int(scratch[:4].view(torch.int32).item()) == 0
