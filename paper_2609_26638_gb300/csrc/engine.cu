@@ -1734,7 +1734,9 @@ int gs_linear(const void* x, const void* w, void* y, int M, int N, int K, int ep
   // A launch of up to 64 rows that is split is shorter than the host's two calls,
   // and a memset is the cheaper of them there (9.3 us a call against 10.2 at 17 x
   // 2048 x 1024); longer launches gain from overlapping their prologue.
-  const bool overlap = p.splits == 1 || M > 64;
+  // (The clear kernel writes words: a scratch that is not aligned to them takes the
+  // memset.)
+  const bool overlap = (p.splits == 1 || M > 64) && (reinterpret_cast<uintptr_t>(scratch) & 3) == 0;
   if ((overlap ? clear_words(static_cast<int*>(scratch), head_bytes / 4, s)
                : cudaMemsetAsync(scratch, 0, head_bytes, s)) != cudaSuccess)
     return GS_ERR_CUDA;

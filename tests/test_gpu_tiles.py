@@ -193,3 +193,24 @@ def test_clusters_above_64_rows(gs, N, K, Ms):
         ref = xm.float() @ w.float().T
         torch.testing.assert_close(y, base[:M] + ref, rtol=1e-4, atol=1e-4 * ref.abs().max().item())
         assert int(scratch[:4].view(torch.int32).item()) == 0
+
+
+@pytest.mark.parametrize("M,split", [(3, 1), (100, 1), (100, 8), (300, 4)])
+@pytest.mark.parametrize("shift", [1, 2])
+def test_linear_takes_a_scratch_at_any_address(gs, M, split, shift):
+    """The scratch has no alignment rule: launches that do not sum partials in it
+    only clear it, and the same bytes come out at any address."""
+    N, K = 1024, 4096
+    g = torch.Generator(device=DEV).manual_seed(M + split)
+    x = torch.randn(M, K, device=DEV, generator=g).half()
+    w = (0.02 * torch.randn(N, K, device=DEV, generator=g)).half()
+    want = torch.zeros(M, N, dtype=torch.float16, device=DEV)
+    _linear(gs, x, w, M, N, K, gs.EPI_STORE_F16, split, want)
+    y = torch.zeros_like(want)
+    sb = gs.gs_linear_scratch_bytes(M, N, split)
+    scratch = torch.full((sb + 4,), 0x7F, dtype=torch.uint8, device=DEV)
+    gs.gs_linear(x.data_ptr(), w.data_ptr(), y.data_ptr(), M, N, K, gs.EPI_STORE_F16, split,
+                 scratch.data_ptr() + shift, sb, torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    assert torch.equal(y, want)
+    assert not scratch[shift:shift + 4].any() and int(scratch[0]) == 0x7F
