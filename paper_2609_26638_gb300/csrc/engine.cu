@@ -1633,9 +1633,9 @@ int gs_attention(int mode, const void* q, const void* kv, int n_pages, const int
   if (rows >= (1ull << 31) || !make_map(&tm, kv, rows, 64, 64)) return GS_ERR_INVALID_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int n_tickets = static_cast<int>(blocks) * n_kv_heads;
-  attn_standalone_prep<<<cdiv(std::max(n_seq * W, n_tickets), 128), 128, 0, s>>>(
-      mode, n, n_seq, W, lim, blk_slot, ticket, n_tickets, err);
-  if (cudaGetLastError() != cudaSuccess) return GS_ERR_CUDA;
+  if (launch_ex(attn_standalone_prep, dim3(cdiv(std::max(n_seq * W, n_tickets), 128)), dim3(128), 0, s,
+                false, dim3(1), mode, n, n_seq, W, lim, blk_slot, ticket, n_tickets, err) != cudaSuccess)
+    return GS_ERR_CUDA;
   AttnArgs a;
   a.q = static_cast<const __half*>(q);
   a.lim = lim;

@@ -11,8 +11,8 @@ static __global__ void clear_words_kernel(int* p, unsigned n) {
 }
 
 cudaError_t clear_words(int* p, size_t n, cudaStream_t s) {
-  clear_words_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, s>>>(p, static_cast<unsigned>(n));
-  return cudaGetLastError();
+  return launch_ex(clear_words_kernel, dim3(static_cast<unsigned>((n + 255) / 256)), dim3(256), 0, s, false,
+                   dim3(1), p, static_cast<unsigned>(n));
 }
 
 template <int BN, int EPI>

@@ -338,3 +338,56 @@ def test_timeout_report_resets_the_merge_tickets(tiny_gain):
     eng.prefill(0, prompt.vis, prompt.text, 40)
     assert decode_all(eng, slots, 8, 40)[0] == before
     eng.close()
+
+
+def test_calls_after_an_earlier_failure(tiny_gain):
+    """A call that failed on the host (a round while its stream is being captured)
+    leaves nothing behind for the calls after it: the attention and the projection
+    judge their own launches only."""
+    from paper_2609_26638_gb300 import gs
+    cfg, w, _ = tiny_gain
+    eng = new_engine(cfg, w, max_ctx=256, max_K=4, max_prefill=128)
+    dev = eng.device
+    o = torch.zeros((1, 8), dtype=torch.int32, device=dev)
+    slots = torch.zeros(1, dtype=torch.int32, device=dev)
+    M, N, K = 100, 256, 256
+    x = torch.randn(M, K, device=dev).half()
+    wl = torch.randn(N, K, device=dev).half()
+    y = torch.zeros(M, N, dtype=torch.float16, device=dev)
+    sl = torch.zeros(gs.gs_linear_scratch_bytes(M, N, 1), dtype=torch.uint8, device=dev)
+    q = torch.randn(1, 5, 8, 64, device=dev).half()
+    kv = torch.randn(2, 2, 4, 64, 64, device=dev).half()
+    pt = torch.tensor([[1, 0]], dtype=torch.int32, device=dev)
+    n = torch.tensor([70], dtype=torch.int32, device=dev)
+    out = torch.zeros_like(q)
+    sa = torch.zeros(gs.gs_attention_scratch_bytes(1, 5, 8, 4, 2, 1), dtype=torch.uint8, device=dev)
+    s = torch.cuda.current_stream(dev).cuda_stream
+
+    def calls():
+        gs.gs_attention(1, q.data_ptr(), kv.data_ptr(), 2, pt.data_ptr(), 2, n.data_ptr(), 1, 5, 8, 4,
+                        out.data_ptr(), sa.data_ptr(), sa.numel(), 1, s)
+        gs.gs_linear(x.data_ptr(), wl.data_ptr(), y.data_ptr(), M, N, K, gs.EPI_STORE_F16, 1,
+                     sl.data_ptr(), sl.numel(), s)
+        torch.cuda.synchronize()
+        return out.clone(), y.clone()
+
+    want = calls()
+
+    def fail():
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.stream(eng.stream):
+            graph.capture_begin(capture_error_mode="thread_local")
+            with pytest.raises(gs.GsError) as e:
+                gs.gs_round(eng.handle, slots.data_ptr(), 1, 2, gs.GS_ACCEPT_GREEDY, None,
+                            o.data_ptr(), o.data_ptr(), o.data_ptr())
+            assert e.value.code == gs.GS_ERR_CUDA
+            graph.capture_end()
+
+    fail()
+    for got, ref in zip(calls(), want):
+        assert torch.equal(got, ref)
+    fail()
+    gs.gs_linear(x.data_ptr(), wl.data_ptr(), y.data_ptr(), M, N, K, gs.EPI_STORE_F16, 1,
+                 sl.data_ptr(), sl.numel(), s)
+    torch.cuda.synchronize()
+    eng.close()
