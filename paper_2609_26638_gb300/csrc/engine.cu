@@ -212,9 +212,9 @@ GemmPlan plan_gemm(int weight_rows, int K, int T, bool decode) {
   return plan_split(weight_rows, T, decode ? decode_splits(weight_rows, K) : 1, K / 64);
 }
 
-// fp32 partials the widest decode tiles (BN > 64, reduced through global
-// scratch) need: splits x feature tiles x token columns (T + 255 bounds the
-// padded token count) x 128, over the decoder's five weight shapes.
+// fp32 partials of the decode windows that reduce through global scratch: splits
+// that form no cluster, which only windows of up to 64 rows (one token tile of 32
+// or 64) take; over the decoder's five weight shapes.
 size_t gemm_partial_floats(const gs_config& c, int qkv_dim, int T_dec) {
   const int HD = c.n_heads * 64;
   const int shapes[5][2] = {{qkv_dim, c.d_model}, {c.d_model, HD}, {2 * c.d_ffn, c.d_model},
@@ -222,8 +222,11 @@ size_t gemm_partial_floats(const gs_config& c, int qkv_dim, int T_dec) {
   size_t need = 0;
   for (const auto& sh : shapes) {
     const int S = decode_splits(sh[0], sh[1]);
-    if (S > 1)
-      need = std::max(need, static_cast<size_t>(S) * (sh[0] / 128) * (T_dec + 255) * 128);
+    for (int T : {std::min(T_dec, 32), std::min(T_dec, 64)}) {
+      const GemmPlan p = plan_split(sh[0], T, S, sh[1] / 64);
+      if (p.splits > 1 && !gemm_cluster_ok(p.bn, p.splits))
+        need = std::max(need, static_cast<size_t>(p.splits) * p.feat_tiles * p.tok_tiles * p.bn * 128);
+    }
   }
   return need;
 }

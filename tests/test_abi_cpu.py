@@ -81,3 +81,24 @@ def test_entry_points_validate_before_launch(gs):
     # cluster split-K (<= 8 splits at <= 64 rows) needs no partials; 32 splits reduce through scratch
     assert gs.gs_linear_scratch_bytes(17, 2048, 8) == gs.gs_linear_scratch_bytes(17, 2048, 1)
     assert gs.gs_linear_scratch_bytes(17, 2048, 32) > gs.gs_linear_scratch_bytes(17, 2048, 1)
+
+
+@pytest.mark.parametrize("d_ffn", [4096, 320])
+def test_workspace_holds_what_its_launches_use(gs, d_ffn):
+    """Serving size (32 sequences, K = 16): the large pieces (KV pool, weight
+    copies, logits, activations, attention rows, rope table) plus at most 32 MiB.
+    Partial sums of split projections exist for splits that form no cluster only
+    (d_ffn 320: five k-blocks, S = 5), for windows of up to 64 rows."""
+    B, ctx, W, d, hq, hkv, V, L = 32, 6720, 17, 1024, 16, 8, 59392, 24
+    cfg = _cfg(gs, n_layers=L, d_model=d, n_heads=hq, n_kv_heads=hkv, d_ffn=d_ffn, vocab=V,
+               mask_token_id=V - 1, max_batch=B, max_ctx=ctx, max_K=W - 1, max_prefill=4096)
+    pages, T = ctx // 64, 4096
+    qkv = (hq + 2 * hkv) * 64
+    kv = L * B * pages * 2 * hkv * 64 * 64 * 2
+    weights = 2 * (L * (qkv * d + d * hq * 64 + 3 * d_ffn * d) + V * d)
+    logits = 2 * B * W * V * 4 + 2 * B * W * (V // 128) * 8
+    acts = T * (4 * d + 2 * d + 4 * (d // 128) + 2 * 2 * hq * 64 + 2 * d_ffn)
+    attn = max(B * 8, -(-T // 64) * 8) * 128 * hkv * 68 * 4
+    rope = ctx * 32 * 8
+    rest = gs.gs_workspace_bytes(cfg) - (kv + weights + logits + acts + attn + rope)
+    assert 0 <= rest <= 32 << 20, rest
