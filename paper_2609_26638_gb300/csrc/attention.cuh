@@ -106,7 +106,7 @@ struct AttnArgs {
   int rows_per_page;          // 2 * Hkv * 64
   int split_pages;            // SP: pages per item
   int max_items;              // items per (block, head) the grid covers
-  int cluster;                // 1: the grid's x dimension is one cluster (max_items <= 16), attn_paged_kernel
+  int cluster;                // 1: attn_paged_kernel, a cluster of max_items (<= 16) CTAs; 0: attn_stream_kernel
   int early;                  // 1: the launch before this one does not write the descriptors or limits
   float* part;                // global merge: [n_blocks][Hkv][max_items][128][kAttnRow]
   int* ticket;                // global merge: [n_blocks][Hkv], zero between launches
@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
   const bool active = s_int[6] != 0;
   const bool bad = maxlim < 0 || npages_blk > a.pt_stride || slot < 0 || nitems > a.max_items ||
                    R > kAttnMaxRows;
-  const bool in_cluster = a.cluster && nitems > 1;
+  const bool in_cluster = nitems > 1;
   if (!active || bad || c >= nitems) {
     if (active && bad && threadIdx.x == 0) atomicExch(a.err, kErrBounds);
     // idle cluster member: counts in the cluster barrier, owns nothing

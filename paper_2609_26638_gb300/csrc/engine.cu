@@ -78,7 +78,6 @@ namespace {
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 inline int cdiv(long long a, long long b) { return static_cast<int>((a + b - 1) / b); }
-inline int round16(int x) { return (x + 15) / 16 * 16; }
 
 // Sequential carving of the caller's workspace (also used to size it).
 struct Carver {
@@ -147,12 +146,11 @@ bool attn_use_cluster(int items, int blocks_x_heads, int rows) {
 
 cudaError_t launch_attention(const CUtensorMap& tm, const AttnArgs& a, int n_blocks,
                              cudaStream_t s, bool pdl) {
-  dim3 grid(a.max_items, a.Hkv, n_blocks);
-  if (!a.cluster)
-    return launch_ex(attn_stream_kernel, dim3(a.Hkv, n_blocks, a.max_items), dim3(kAttnThreads), kAttnStreamSmem, s, pdl,
-                     dim3(1, 1, 1), tm, a);
-  return launch_ex(attn_paged_kernel, grid, dim3(kAttnThreads), kAttnSmemBytes, s, pdl,
-                   dim3(a.cluster ? a.max_items : 1, 1, 1), tm, a);
+  if (a.cluster)
+    return launch_ex(attn_paged_kernel, dim3(a.max_items, a.Hkv, n_blocks), dim3(kAttnThreads), kAttnSmemBytes,
+                     s, pdl, dim3(a.max_items, 1, 1), tm, a);
+  return launch_ex(attn_stream_kernel, dim3(a.Hkv, n_blocks, a.max_items), dim3(kAttnThreads),
+                   kAttnStreamSmem, s, pdl, dim3(1, 1, 1), tm, a);
 }
 
 struct GemmPlan {
@@ -255,7 +253,7 @@ struct gs_handle {
   // sizes
   int qkv_dim = 0, G = 1, T_max = 0, pt_stride = 0, n_pages = 0, W_max = 1;
   // attention work items: pages per item and item slots, decode and prefill
-  int split_pages = 1, items_dec = 1, r_max_dec = 16;
+  int split_pages = 1, items_dec = 1;
   int split_pages_pf = 8, items_pf = 1, qb_pf = 64;
   float* attn_part = nullptr;
   size_t attn_part_floats = 0;
@@ -393,7 +391,6 @@ size_t carve(gs_handle* h, const gs_config& c, void* base) {
   // items per sequence (one cluster) when a full batch of them still fits in
   // about one wave of CTAs, else at most 8, unless the config asks for
   // smaller items; prefill: at least 8 pages per item, at most 8 items.
-  const int r_max = round16(W_max * G);
   const AttnGeom g_dec = attn_geom(W_max, G);
   const int qb_pf = std::max(1, kAttnMaxRows / G);
   const int items_target =
@@ -475,7 +472,6 @@ size_t carve(gs_handle* h, const gs_config& c, void* base) {
     h->W_max = W_max;
     h->split_pages = sp;
     h->items_dec = items_dec;
-    h->r_max_dec = r_max;
     h->split_pages_pf = sp_pf;
     h->items_pf = items_pf;
     h->qb_pf = qb_pf;

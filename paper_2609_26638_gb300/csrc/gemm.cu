@@ -49,7 +49,9 @@ static cudaError_t launch_bn(int epi, const CUtensorMap& tmW, const CUtensorMap&
     case kEpiResidF32: return launch_one<BN, kEpiResidF32>(tmW, tmX, a, ft, tt, s, pdl);
     case kEpiSwiGLU: return launch_one<BN, kEpiSwiGLU>(tmW, tmX, a, ft, tt, s, pdl);
     case kEpiArgmax: return launch_one<BN, kEpiArgmax>(tmW, tmX, a, ft, tt, s, pdl);
-    case kEpiQKV: return launch_one<BN, kEpiQKV>(tmW, tmX, a, ft, tt, s, pdl);
+    case kEpiQKV:   // the decoder's own launches: tiles of 32 and 64
+      if constexpr (BN <= 64) return launch_one<BN, kEpiQKV>(tmW, tmX, a, ft, tt, s, pdl);
+      break;
   }
   return cudaErrorInvalidValue;
 }
@@ -83,8 +85,9 @@ static cudaError_t set_attr_bn() {
   if ((e = cudaFuncSetAttribute(gemm_tc_kernel<BN, kEpiArgmax>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess)
     return e;
-  return cudaFuncSetAttribute(gemm_tc_kernel<BN, kEpiQKV>,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if constexpr (BN <= 64)
+    e = cudaFuncSetAttribute(gemm_tc_kernel<BN, kEpiQKV>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  return e;
 }
 
 cudaError_t gemm_init_attributes() {
