@@ -323,6 +323,7 @@ struct gs_handle {
 namespace {
 
 int fail(gs_handle* h, int code, const std::string& msg) {
+  if (code == GS_ERR_CUDA) cudaGetLastError();   // reported here: nothing left for the next call to find
   if (h) h->err = msg;
   else g_create_error = msg;
   return code;

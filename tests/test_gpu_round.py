@@ -391,3 +391,26 @@ def test_calls_after_an_earlier_failure(tiny_gain):
                  sl.data_ptr(), sl.numel(), s)
     torch.cuda.synchronize()
     eng.close()
+
+
+def test_engine_after_an_earlier_failure(tiny_gain):
+    """The same for the calls of a decoder: one is built and prefilled after a round
+    that could not be captured."""
+    from paper_2609_26638_gb300 import gs
+    cfg, w, _ = tiny_gain
+    eng = new_engine(cfg, w, max_ctx=256, max_K=4, max_prefill=128)
+    o = torch.zeros((1, 8), dtype=torch.int32, device=eng.device)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(eng.stream):
+        graph.capture_begin(capture_error_mode="thread_local")
+        with pytest.raises(gs.GsError) as e:
+            gs.gs_round(eng.handle, o.data_ptr(), 1, 2, gs.GS_ACCEPT_GREEDY, None, o.data_ptr(),
+                        o.data_ptr(), o.data_ptr())
+        assert e.value.code == gs.GS_ERR_CUDA and "Capture" in str(e.value)
+        graph.capture_end()
+    p = synth.make_prompt(cfg, 20, 5, index=1)
+    x0 = eng.prefill(0, p.vis, p.text, 8)
+    other = new_engine(cfg, w, max_ctx=256, max_K=4, max_prefill=128)
+    assert other.prefill(0, p.vis, p.text, 8) == x0
+    eng.close()
+    other.close()
