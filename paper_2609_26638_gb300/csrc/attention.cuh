@@ -33,7 +33,8 @@
 // Merge over items, item order 0, 1, ...: M = max m_i, w_i = exp2(m_i - M),
 // coef_i = w_i / sum_j w_j l_j, O = sum coef_i O_i.  A block with one item
 // writes its rows directly.  The kernel of this file is for small launches (at
-// most 16 items per (block, head), about one wave of CTAs): the items of a
+// most 16 items per (block, head), about one wave of CTAs; two waves for at most
+// eight items of more than 96 rows): the items of a
 // (block, head) form a thread-block cluster, and once every CTA of it has
 // finished its pages, each sends the rows that CTA (r mod n) owns to it with one
 // bulk async copy into its shared memory, completing on its mbarrier, and each

@@ -10,9 +10,11 @@
 // it drops the CTAs whose item lies past the sequence's end: with a CTA per
 // item, each paid 1.5 us of start-up, 0.9 us for Q and 2.5-3 us for its rows and
 // ticket around 8 us of pages (13 pages of a 17-token window, 1.5 of 2 CTAs
-// resident).  64 sequences of 8192 keys take 206 us (290 with a CTA per item), a
-// prefill chunk of 1024 tokens 78 (98); 32 sequences of 1-6 k keys take the same.
-// The arithmetic and its order are attention.cuh's.
+// resident).  With the same page loop, 64 sequences of 8192 keys took 227 us with
+// a CTA per item and 207 here, a prefill chunk of 1024 tokens 85.5 and 78, 32
+// sequences of 1-6 k keys 80 and 81; with the merges' loads in flight together
+// (attn_merge_rows) 195, 63.6 and 71.7.  The arithmetic and its order are
+// attention.cuh's.
 //
 // Warps 0-3: softmax, the item's rows to global scratch, and merges; 4: producer
 // (scheduling, descriptors, page copies, tickets); 5: MMA issue.  An item's rows
@@ -482,7 +484,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
     }
   } else {
     // ---- softmax warps.  An item's descriptor stays in its slot until its rows
-    // are out (registers are short: 128 a thread with two CTAs of seven warps).
+    // are out (registers are short: 168 a thread with two CTAs of six warps).
     AttnSync y{s_full, s_free, p_full, v_empty, sP, m_row};
     AttnRings rg;
     RingPos ws;

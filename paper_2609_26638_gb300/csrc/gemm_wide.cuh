@@ -32,8 +32,9 @@
 // clock and SM from L2; 350 at 144; 515 at 256, which is the MMA rate).  One
 // CTA per tile instead paid its start-up, its first load latency and its
 // epilogue per tile: 544 rows of gate/up took 24.5 us, LM head at 17 rows 30 us,
-// a 4096-row prefill gate/up 100 us; here 18.5, 27.0 (23.6 as a graph node, 76% of
-// the measured copy rate) and 57-60 us.
+// a 4096-row prefill gate/up 100 us; here 19.0, 26.6 (23.6 as a graph node, 76% of
+// the measured copy rate) and 57-59 us.  (The 256-row residual kernel spills 32
+// bytes beyond its 168 registers; the others none.)
 #pragma once
 #include "gemm_tc.cuh"
 
