@@ -1731,9 +1731,10 @@ int gs_linear(const void* x, const void* w, void* y, int M, int N, int K, int ep
   a.logits = nullptr;
   a.w_scale = 1.f;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // A launch of up to 64 rows that is split is shorter than the host's two calls,
-  // and a memset is the cheaper of them there (9.3 us a call against 10.2 at 17 x
-  // 2048 x 1024); longer launches gain from overlapping their prologue.
+  // A split launch of up to 64 rows follows a memset (9.3 us a call against 10.2 with
+  // the clear kernel, back to back at 17 x 2048 x 1024; the host takes 2.9 of them:
+  // 0.1 per tensor map, 0.9 the memset, 1.8 the launch); longer launches gain from
+  // overlapping their prologue.
   // (The clear kernel writes words: a scratch that is not aligned to them takes the
   // memset.)
   const bool overlap = (p.splits == 1 || M > 64) && (reinterpret_cast<uintptr_t>(scratch) & 3) == 0;
