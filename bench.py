@@ -70,13 +70,13 @@ def schedule_rounds(sched: np.ndarray, max_new: int) -> int:
 _CSRC = os.path.join(ROOT, "paper_2609_26638_gb300", "csrc")
 NCU_TRAFFIC = {
     "attention_b1": dict(sources=("attention.cuh", "ptx.cuh"), bytes=4934144, algorithmic=4823040,
-                         sha256="a3a681e67936a67131bf0807979510cab74ae62f207601b15016df7419539d75"),
+                         sha256="fcf89da96323a3a2d00a94b413726e715cbc6066eaf67e9db2f40475c1fab9a4"),
     "attention_serve": dict(sources=("attention.cuh", "attention_stream.cuh", "ptx.cuh"),
-                            bytes=233422592, algorithmic=225173504,
-                            sha256="ba0eda31823029a4f665c31dcefd451641439a391145d9c15ef25ef69d703305"),
+                            bytes=233444352, algorithmic=225173504,
+                            sha256="fc17e03133f39c4609f54fbf998e3f918ea503e4d84ec63e708dc39ecaa6ba7d"),
     "lm_head_b1": dict(sources=("gemm_tc.cuh", "gemm_wide.cuh", "gemm_wide.cu", "ptx.cuh"),
-                       bytes=124454144, algorithmic=121669768,
-                       sha256="239775d170ba9d4ae12d02bf55c93c86d37f5d8ac676b82c75a59f28efbb164f"),
+                       bytes=124607744, algorithmic=121669768,
+                       sha256="eabd23cf7a5c44b0d6dee526756fe7a54220d3439125dd7d591f85f4695422c3"),
 }
 
 
