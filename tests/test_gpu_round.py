@@ -414,3 +414,25 @@ def test_engine_after_an_earlier_failure(tiny_gain):
     assert other.prefill(0, p.vis, p.text, 8) == x0
     eng.close()
     other.close()
+
+
+def test_wide_model_batch_equals_single():
+    """d_model 4096: the QKV projection's split forms clusters of eight also above 64
+    rows.  Eight sequences in one batch (136 rows) commit what each commits alone
+    (17 rows, and 17-row windows are in lock-step with the oracle)."""
+    cfg = synth.TINY.with_(n_layers=1, d_model=4096, n_heads=8, n_kv_heads=4)
+    w = synth.make_weights(cfg, seed=13)
+    K, B, cap = 16, 8, 24
+    eng = new_engine(cfg, w, max_batch=B, max_ctx=256, max_K=K, max_prefill=128)
+    prompts = [synth.make_prompt(cfg, 20 + 9 * i, 5, index=60 + i) for i in range(B)]
+    st, stats = lockstep(eng, Decoder(cfg, w), prompts[0], K, cap, check_logits=True)
+    assert st.done
+    single = []
+    for i, p in enumerate(prompts):
+        eng.prefill(i, p.vis, p.text, cap)
+        single.append(decode_all(eng, torch.tensor([i], dtype=torch.int32, device=eng.device), K, 40)[0])
+    for i, p in enumerate(prompts):
+        eng.prefill(i, p.vis, p.text, cap)
+    slots = torch.arange(B, dtype=torch.int32, device=eng.device)
+    assert decode_all(eng, slots, K, 40) == single
+    eng.close()

@@ -214,3 +214,25 @@ def test_linear_takes_a_scratch_at_any_address(gs, M, split, shift):
     torch.cuda.synchronize()
     assert torch.equal(y, want)
     assert not scratch[shift:shift + 4].any() and int(scratch[0]) == 0x7F
+
+
+@pytest.mark.parametrize("epi,N", [(0, 1024), (2, 1024), (3, 2048)])
+def test_clusters_above_64_rows_other_epilogues(gs, epi, N):
+    """fp16 stores, SwiGLU and argmax keys of 100 rows in clusters of eight (at most
+    256 CTAs): every row has the bits it has alone in a window of its own 17."""
+    M, K = 100, 4096
+    g = torch.Generator(device=DEV).manual_seed(epi)
+    x = torch.randn(M, K, device=DEV, generator=g).half()
+    w = (0.02 * torch.randn(2 * N if epi == gs.EPI_SWIGLU else N, K, device=DEV, generator=g)).half()
+
+    def out(m):
+        return (torch.zeros(m, dtype=torch.int64, device=DEV) if epi == gs.EPI_ARGMAX
+                else torch.zeros(m, N, dtype=torch.float16, device=DEV))
+
+    y = out(M)
+    _linear(gs, x, w, M, N, K, epi, 8, y)
+    for m0 in range(0, M, 17):
+        m = min(17, M - m0)
+        part = out(m)
+        _linear(gs, x[m0:m0 + m].contiguous(), w, m, N, K, epi, 8, part)
+        assert torch.equal(y[m0:m0 + m], part), m0
