@@ -109,7 +109,7 @@ struct AttnArgs {
   int max_items;              // items per (block, head) the grid covers
   int cluster;                // 1: attn_paged_kernel, a cluster of max_items (<= 16) CTAs; 0: attn_stream_kernel
   int early;                  // 1: the launch before this one does not write the descriptors or limits
-  float* part;                // global merge: [n_blocks][Hkv][max_items][128][kAttnRow]
+  float* part;                // global merge: [n_blocks][Hkv][max_items] tiles of 128 * kAttnRow floats
   int* ticket;                // global merge: [n_blocks][Hkv], zero between launches
   int* err;
 };

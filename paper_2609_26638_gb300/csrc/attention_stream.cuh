@@ -13,7 +13,7 @@
 // resident).  With the same page loop, 64 sequences of 8192 keys took 227 us with
 // a CTA per item and 207 here, a prefill chunk of 1024 tokens 85.5 and 78, 32
 // sequences of 1-6 k keys 80 and 81; with the merges' loads in flight together
-// (attn_merge_rows) 195, 63.6 and 71.7.  The arithmetic and its order are
+// (attn_merge_rows) 194, 57.5 and 69.  The arithmetic and its order are
 // attention.cuh's.
 //
 // Warps 0-3: softmax, the item's rows to global scratch, and merges; 4: producer
@@ -35,6 +35,11 @@ constexpr int kAttnStreamTail = 512;
 constexpr int kAttnStreamSmem = 1024 + kAttnBarOff + kAttnStreamTail + kAttnMaxRows * 4 + kAttnPtAhead * 4;
 static_assert(2 * (kAttnStreamSmem + 1024) <= 228 * 1024, "two CTAs per SM");
 
+// An item's rows in global scratch: O [128][64], then (m, l) [128] -- whole 128-byte
+// lines of O, and one line of (m, l) for 16 rows, where the merge reads them.
+constexpr int kAttnTileMl = kAttnMaxRows * 64;
+static_assert(kAttnTileMl + 2 * kAttnMaxRows <= kAttnMaxRows * kAttnRow, "the tile holds rows and (m, l)");
+
 struct AttnWork {
   int np, p_begin, nitems, tok0, R, b, h, c;   // np == 0: no more work
 };
@@ -46,9 +51,11 @@ struct AttnWork {
 // two at a time: the rows come from L2, so loads in flight decide, and a launch
 // ends with merges that nothing overlaps (two per CTA at worst).  The loads are
 // unconditional and stand before a __syncwarp: with a condition on each, the
-// compiler put every load beside its use, eight round trips in a row (rows of 8
-// items: 14.3 us for 98 rows, 5.4 for 34; now 5.7 and 2.7.  5 sequences x 6000
-// slots, 49 tokens: 75 us a launch, now 50; CTAs for one item each took 53).
+// compiler put every load beside its use, eight round trips in a row.  A merge of
+// 98 rows of 8 items took 16.6 us so, 5.8 now; of 34 rows 7.1 and 3.6; of 10 rows
+// of 27 items 12.2 (four loads of (m, l) at a time) and 6.5.  Launches: 10 windows
+// of 49 tokens at 6000 slots 90.5 us so, 61.7 now (73 with a CTA per item), one
+// window of 5 tokens at 8000 slots in 26 items 25.3 and 19.5 (21.4).
 // `bar` completes two phases per merge: coefficients written, and read (the P
 // tiles are the softmax's again).  False if a wait ran out.
 __device__ __forceinline__ bool attn_merge_rows(const float* part, float* coef, __half* out, uint64_t* bar,
@@ -56,11 +63,13 @@ __device__ __forceinline__ bool attn_merge_rows(const float* part, float* coef, 
                                              int g_magic, int* err) {
   constexpr int kUnits = 2;
   const size_t step = static_cast<size_t>(kAttnMaxRows) * kAttnRow;   // item to item
-  if (threadIdx.x < R) {
-    const float* row = part + static_cast<size_t>(threadIdx.x) * kAttnRow + 64;
-    float* cf = coef + threadIdx.x;
-    float M = -INFINITY, L = 0.f;
-    if (nitems <= 8) {
+  const int r = min(static_cast<int>(threadIdx.x), R - 1);
+  const bool own = threadIdx.x < R;
+  const float* row = part + kAttnTileMl + 2 * r;
+  float* cf = coef + r;
+  float M = -INFINITY, L = 0.f;
+  if (nitems <= 8) {
+    if (own) {
       float2 ml[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u)
@@ -78,18 +87,40 @@ __device__ __forceinline__ bool attn_merge_rows(const float* part, float* coef, 
 #pragma unroll
       for (int u = 0; u < 8; ++u)
         if (u < nitems) cf[u * kAttnMaxRows] = ml[u].x * inv;
-    } else {
-#pragma unroll 4
-      for (int it = 0; it < nitems; ++it) M = fmaxf(M, __ldcg(row + it * step));
-#pragma unroll 4
-      for (int it = 0; it < nitems; ++it) {
-        const float2 ml = __ldcg(reinterpret_cast<const float2*>(row + it * step));
-        const float w = ml.x == -INFINITY ? 0.f : exp2f(ml.x - M);
-        cf[it * kAttnMaxRows] = w;
-        L += w * ml.y;
-      }
-      const float inv = 1.0f / L;
+    }
+  } else if (static_cast<int>(threadIdx.x & ~31u) < R) {   // (warp-uniform)
+    // sixteen loads in flight: the maxima, kept in the coefficients' places, then
+    // the sums
 #pragma unroll 1
+    for (int it0 = 0; it0 < nitems; it0 += 16) {
+      float v[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) v[u] = __ldcg(row + min(it0 + u, nitems - 1) * step);
+      __syncwarp();
+#pragma unroll
+      for (int u = 0; u < 16; ++u) M = fmaxf(M, v[u]);   // (a repeated item changes no maximum)
+#pragma unroll
+      for (int u = 0; u < 16; ++u)
+        if (own && it0 + u < nitems) cf[(it0 + u) * kAttnMaxRows] = v[u];
+    }
+#pragma unroll 1
+    for (int it0 = 0; it0 < nitems; it0 += 16) {
+      float v[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) v[u] = __ldcg(row + 1 + min(it0 + u, nitems - 1) * step);
+      __syncwarp();
+#pragma unroll
+      for (int u = 0; u < 16; ++u)
+        if (own && it0 + u < nitems) {
+          float* c = cf + (it0 + u) * kAttnMaxRows;
+          const float w = *c == -INFINITY ? 0.f : exp2f(*c - M);
+          *c = w;
+          L += w * v[u];
+        }
+    }
+    const float inv = 1.0f / L;
+    if (own) {
+#pragma unroll 4
       for (int it = 0; it < nitems; ++it) cf[it * kAttnMaxRows] *= inv;
     }
   }
@@ -104,13 +135,13 @@ __device__ __forceinline__ bool attn_merge_rows(const float* part, float* coef, 
     const int idx = base + (threadIdx.x & 31);
     float4 acc[kUnits];
     const float* src[kUnits];
-    const float* cf[kUnits];
+    const float* w_of[kUnits];
 #pragma unroll
     for (int q = 0; q < kUnits; ++q) {
       const int i = min(idx + q * kAttnSoftThreads, R * 16 - 1);
       acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-      src[q] = part + static_cast<size_t>(i >> 4) * kAttnRow + (i & 15) * 4;
-      cf[q] = coef + (i >> 4);
+      src[q] = part + i * 4;
+      w_of[q] = coef + (i >> 4);
     }
 #pragma unroll 1
     for (int it0 = 0; it0 < nitems; it0 += 8) {
@@ -129,7 +160,7 @@ __device__ __forceinline__ bool attn_merge_rows(const float* part, float* coef, 
         const int it = min(it0 + u, nitems - 1);
 #pragma unroll
         for (int q = 0; q < kUnits; ++q) {
-          const float w = cf[q][it * kAttnMaxRows];
+          const float w = w_of[q][it * kAttnMaxRows];
           acc[q].x = live ? acc[q].x + w * v[q][u].x : acc[q].x;
           acc[q].y = live ? acc[q].y + w * v[q][u].y : acc[q].y;
           acc[q].z = live ? acc[q].z + w * v[q][u].z : acc[q].z;
@@ -539,11 +570,12 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
         part = a.part + (static_cast<size_t>(w.b) * a.Hkv + w.h) * a.max_items * kAttnMaxRows * kAttnRow;
         if (r < w.R) {
           if (post) {
-            float* dst = part + (static_cast<size_t>(w.c) * kAttnMaxRows + r) * kAttnRow;
+            float* tile = part + static_cast<size_t>(w.c) * kAttnMaxRows * kAttnRow;
+            float* dst = tile + r * 64;
 #pragma unroll
             for (int k = 0; k < 64; k += 4)
               *reinterpret_cast<float4*>(dst + k) = make_float4(O(k), O(k + 1), O(k + 2), O(k + 3));
-            *reinterpret_cast<float2*>(dst + 64) = make_float2(m_row[threadIdx.x], l);
+            *reinterpret_cast<float2*>(tile + kAttnTileMl + 2 * r) = make_float2(m_row[threadIdx.x], l);
           } else {   // the block's only item: its rows are final
             const float inv = 1.0f / l;
             const int tt = r * a.g_magic >> 16;

@@ -137,8 +137,8 @@ namespace {
 // clusters fragment larger grids); otherwise through global scratch.  Both
 // give the same bits.  Blocks of more than 96 rows stay in (portable) clusters
 // up to two waves: there a merge of up to 128 rows by one CTA is the longer
-// tail (305-608 CTAs, 100-8000 slots: persistent / cluster time 0.87-1.87, 1.12
-// in the mean; at 66 rows 0.86-1.26, 1.03; above 608 CTAs ragged batches lose).
+// tail (305-608 CTAs, 100-8000 slots: persistent / cluster time 0.82-1.99, 1.15
+// in the mean; at up to 96 rows they are even; above 608 CTAs ragged batches lose).
 bool attn_use_cluster(int items, int blocks_x_heads, int rows) {
   const int waves = rows > 96 && items <= kMaxClusterSplits ? 2 : 1;
   return items <= kAttnMaxCluster && items * blocks_x_heads <= waves * 2 * kNumSMs;

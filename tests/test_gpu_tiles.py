@@ -236,3 +236,23 @@ def test_clusters_above_64_rows_other_epilogues(gs, epi, N):
         part = out(m)
         _linear(gs, x[m0:m0 + m].contiguous(), w, m, N, K, epi, 8, part)
         assert torch.equal(y[m0:m0 + m], part), m0
+
+
+@pytest.mark.parametrize("items", [9, 16, 17, 32, 33, 54])
+@pytest.mark.parametrize("W,Hq,Hkv", [(5, 16, 8), (16, 16, 2)])
+def test_attention_merges_many_items(gs, items, W, Hq, Hkv):
+    """One-page items beyond eight, up to the interface's 54, merged through global
+    scratch: their maxima and sums are read sixteen at a time (blocks of 10 and of
+    128 rows)."""
+    B = 40 if Hkv == 2 else 6                  # more than one wave of CTAs
+    rng = np.random.default_rng(items)
+    ns = [64 * items - 40] + [int(v) for v in rng.integers(1, 64 * items - 40, B - 1)]
+    q, k, v = synth.attn_inputs(B, W, 64 * items, Hq, Hkv, index=items)
+    pool, pt, _ = _paged(k, v, rng)
+    got = _run_attention(gs, 1, q, pool, pt, np.array(ns), W, Hq, Hkv, 1)
+    for b in (0, 1, int(np.argmin(ns))):
+        allowed = od.verify_allowed(ns[b], W - 1)
+        nk = allowed.shape[1]
+        want = _oracle_attn(q[b].astype(np.float64), k[b, :nk].astype(np.float64),
+                            v[b, :nk].astype(np.float64), allowed, Hq, Hkv)
+        np.testing.assert_allclose(got[b], want, rtol=5e-3, atol=5e-3)
