@@ -36,9 +36,13 @@ static cudaError_t launch_one(const CUtensorMap& tmW, const CUtensorMap& tmX, Ge
   const int kb = a.kb_per_split;
   a.stages = kb < S::kStagesMin ? S::kStagesMin : (kb > want ? want : kb);
   dim3 grid(tok_tiles, feat_tiles, a.splits);
-  const int cz = cl ? a.splits : 1;
-  return launch_ex(gemm_tc_kernel<BN, EPI>, grid, dim3(128), S::smem_bytes(a.stages, EPI, cl), s,
-                   pdl, dim3(1, 1, cz), tmW, tmX, a);
+  const size_t smem = S::smem_bytes(a.stages, EPI, cl);
+  if constexpr (S::kClusterOk) {
+    if (cl)
+      return launch_ex(gemm_tc_kernel<BN, EPI, true>, grid, dim3(128), smem, s, pdl, dim3(1, 1, a.splits), tmW,
+                       tmX, a);
+  }
+  return launch_ex(gemm_tc_kernel<BN, EPI, false>, grid, dim3(128), smem, s, pdl, dim3(1, 1, 1), tmW, tmX, a);
 }
 
 template <int BN>
@@ -69,24 +73,25 @@ cudaError_t launch_gemm(int bn, int epi, const CUtensorMap& tmW, const CUtensorM
   return cudaErrorInvalidValue;
 }
 
+template <int BN, int EPI>
+static cudaError_t set_attr_one() {
+  cudaError_t e = cudaSuccess;
+  if constexpr (GemmShape<BN>::kClusterOk)
+    e = cudaFuncSetAttribute(gemm_tc_kernel<BN, EPI, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             GemmShape<BN>::kSmemMax);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(gemm_tc_kernel<BN, EPI, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              GemmShape<BN>::kSmemMax);
+}
+
 template <int BN>
 static cudaError_t set_attr_bn() {
-  const int bytes = GemmShape<BN>::kSmemMax;
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(gemm_tc_kernel<BN, kEpiStoreF16>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess)
-    return e;
-  if ((e = cudaFuncSetAttribute(gemm_tc_kernel<BN, kEpiResidF32>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess)
-    return e;
-  if ((e = cudaFuncSetAttribute(gemm_tc_kernel<BN, kEpiSwiGLU>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess)
-    return e;
-  if ((e = cudaFuncSetAttribute(gemm_tc_kernel<BN, kEpiArgmax>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess)
-    return e;
-  if constexpr (BN <= 64)
-    e = cudaFuncSetAttribute(gemm_tc_kernel<BN, kEpiQKV>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if ((e = set_attr_one<BN, kEpiStoreF16>()) != cudaSuccess) return e;
+  if ((e = set_attr_one<BN, kEpiResidF32>()) != cudaSuccess) return e;
+  if ((e = set_attr_one<BN, kEpiSwiGLU>()) != cudaSuccess) return e;
+  if ((e = set_attr_one<BN, kEpiArgmax>()) != cudaSuccess) return e;
+  if constexpr (BN <= 64) e = set_attr_one<BN, kEpiQKV>();
   return e;
 }
 

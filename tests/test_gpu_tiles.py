@@ -256,3 +256,35 @@ def test_attention_merges_many_items(gs, items, W, Hq, Hkv):
         want = _oracle_attn(q[b].astype(np.float64), k[b, :nk].astype(np.float64),
                             v[b, :nk].astype(np.float64), allowed, Hq, Hkv)
         np.testing.assert_allclose(got[b], want, rtol=5e-3, atol=5e-3)
+
+
+@pytest.mark.parametrize("N,K,split", [(256, 640, 5), (512, 1216, 19), (384, 2048, 32)])
+@pytest.mark.parametrize("epi", [0, 1, 3])
+def test_split_sums_through_scratch(gs, N, K, split, epi):
+    """Splits that form no cluster, around the slices of 8 and 32 tokens in which the
+    last CTA adds them up, with the splits' remainders: a row's bits are those of the
+    64-row window, and the allocation-free call's tiles of up to 256 rows give the
+    same."""
+    g = torch.Generator(device=DEV).manual_seed(N + split)
+    x = torch.randn(137, K, device=DEV, generator=g).half()
+    w = (0.05 * torch.randn(N, K, device=DEV, generator=g)).half()
+    base = torch.randn(137, N, device=DEV, generator=g)
+
+    def out(m):
+        if epi == gs.EPI_RESID_F32:
+            return base[:m].clone()
+        return (torch.zeros(m, dtype=torch.int64, device=DEV) if epi == gs.EPI_ARGMAX
+                else torch.zeros(m, N, dtype=torch.float16, device=DEV))
+
+    want = out(137)
+    _linear(gs, x, w, 137, N, K, epi, split, want)     # chunks inside each CTA
+    for M in (1, 7, 8, 9, 32, 33, 40, 41, 64):
+        y = out(M)
+        _linear(gs, x[:M].contiguous(), w, M, N, K, epi, split, y)
+        assert torch.equal(y, want[:M]), M
+    stream = torch.cuda.current_stream().cuda_stream
+    for M in (8, 9, 72, 73) + ((136, 137) if split == 5 else ()):   # (partials within 8 MiB)
+        xm, y = x[:M].contiguous(), out(M)
+        gs.gs_linear_noalloc(xm.data_ptr(), w.data_ptr(), y.data_ptr(), M, N, K, epi, split, stream)
+        assert gs.gs_linear_noalloc_status(stream) == gs.GS_OK
+        assert torch.equal(y, want[:M]), M
