@@ -188,7 +188,7 @@ int decode_splits(int weight_rows, int K) {
 // 2048 x 8192 13.4 / 22.0 at 65, 21.0 / 21.9 at 129; 256 x 4096 7.2 / 13.3 at 65,
 // 9.5 / 14.1 at 544.  Clusters of 4 stay below one wave's worth of gain (4096 x
 // 2048: 11.3 / 9.9 at 128 rows, 4096 x 4096 14.1 / 14.0).
-GemmPlan plan_split(int weight_rows, int T, int S, int nkb) {
+GemmPlan plan_split(int epi, int weight_rows, int T, int S, int nkb) {
   GemmPlan p;
   p.feat_tiles = weight_rows / 128;
   const bool clusters = S == kMaxClusterSplits && nkb / S >= 8 &&
@@ -200,14 +200,14 @@ GemmPlan plan_split(int weight_rows, int T, int S, int nkb) {
   } else {
     p.splits = 1;
     p.chunks = S;
-    p.bn = wide_bn(p.feat_tiles, T, nkb);
+    p.bn = unsplit_bn(epi, p.feat_tiles, T, nkb, S);
   }
   p.tok_tiles = cdiv(T, p.bn);
   return p;
 }
 
-GemmPlan plan_gemm(int weight_rows, int K, int T, bool decode) {
-  return plan_split(weight_rows, T, decode ? decode_splits(weight_rows, K) : 1, K / 64);
+GemmPlan plan_gemm(int epi, int weight_rows, int K, int T, bool decode) {
+  return plan_split(epi, weight_rows, T, decode ? decode_splits(weight_rows, K) : 1, K / 64);
 }
 
 // fp32 partials of the decode windows that reduce through global scratch: splits
@@ -221,7 +221,7 @@ size_t gemm_partial_floats(const gs_config& c, int qkv_dim, int T_dec) {
   for (const auto& sh : shapes) {
     const int S = decode_splits(sh[0], sh[1]);
     for (int T : {std::min(T_dec, 32), std::min(T_dec, 64)}) {
-      const GemmPlan p = plan_split(sh[0], T, S, sh[1] / 64);
+      const GemmPlan p = plan_split(kEpiStoreF16, sh[0], T, S, sh[1] / 64);
       if (p.splits > 1 && !gemm_cluster_ok(p.bn, p.splits))
         need = std::max(need, static_cast<size_t>(p.splits) * p.feat_tiles * p.tok_tiles * p.bn * 128);
     }
@@ -247,7 +247,7 @@ struct gs_handle {
   __half* wcopy = nullptr;
   std::vector<CUtensorMap> tm_qkv, tm_o, tm_gu, tm_down;
   CUtensorMap tm_lm;
-  CUtensorMap tm_hb[kWideTiles], tm_ao[kWideTiles], tm_act[kWideTiles];
+  CUtensorMap tm_hb[kTokenMaps], tm_ao[kTokenMaps], tm_act[kTokenMaps];
   CUtensorMap tm_kv;
 
   // sizes
@@ -539,7 +539,7 @@ GemmArgs gemm_base(gs_handle* h) {
 
 int run_gemm(gs_handle* h, const CUtensorMap& tw, int weight_rows, const CUtensorMap* tx_set, int K,
              int T, int epi, GemmArgs a, bool decode, int kind) {
-  const GemmPlan p = plan_gemm(weight_rows, K, T, decode);
+  const GemmPlan p = plan_gemm(epi, weight_rows, K, T, decode);
   a.M = T;
   a.K = K;
   a.splits = p.splits;
@@ -550,7 +550,7 @@ int run_gemm(gs_handle* h, const CUtensorMap& tw, int weight_rows, const CUtenso
       (static_cast<size_t>(p.splits) * p.feat_tiles * p.tok_tiles * p.bn * 128 > h->partial_floats ||
        p.feat_tiles * p.tok_tiles > kGemmCounters))
     return fail(h, GS_ERR_OOM, "split-K scratch too small");
-  GS_CUDA(h, launch_gemm(p.bn, epi, tw, tx_set[wide_index(p.bn)], a, p.feat_tiles, p.tok_tiles,
+  GS_CUDA(h, launch_gemm(p.bn, epi, tw, tx_set[token_map_index(p.bn)], a, p.feat_tiles, p.tok_tiles,
                          h->stream, h->pdl));
   note_launch(h, kind);
   return GS_OK;
@@ -1127,10 +1127,10 @@ int gs_create(const gs_config* cfg, const gs_weights* w, void* workspace, size_t
          make_map_swiglu(&h->tm_gu[l], h->w_gu[l], F, d) &&
          make_map(&h->tm_down[l], h->w_down[l], d, F, 128);
   ok = ok && make_map(&h->tm_lm, h->lm_head, c.vocab, d, 128);
-  for (int i = 0; i < kWideTiles && ok; ++i) {
-    ok = make_map(&h->tm_hb[i], h->hb, h->T_max, d, kWideBN[i]) &&
-         make_map(&h->tm_ao[i], h->ao, h->T_max, HD, kWideBN[i]) &&
-         make_map(&h->tm_act[i], h->act, h->T_max, F, kWideBN[i]);
+  for (int i = 0; i < kTokenMaps && ok; ++i) {
+    ok = make_map(&h->tm_hb[i], h->hb, h->T_max, d, kTokenMapBN[i]) &&
+         make_map(&h->tm_ao[i], h->ao, h->T_max, HD, kTokenMapBN[i]) &&
+         make_map(&h->tm_act[i], h->act, h->T_max, F, kTokenMapBN[i]);
   }
   const uint64_t kv_rows = static_cast<uint64_t>(L) * h->n_pages * 2 * c.n_kv_heads * 64;
   ok = ok && kv_rows < (1ull << 31) && make_map(&h->tm_kv, h->kv, kv_rows, 64, 64);
@@ -1673,7 +1673,7 @@ size_t gs_linear_scratch_bytes(int M, int N, int split_k) {
   // no cluster; launches over 64 rows split K inside a CTA or a cluster and use neither
   size_t counters = 0, partial = 0;
   for (int w_rows : {N, 2 * N}) {
-    const GemmPlan p = plan_split(w_rows, M, split_k, split_k);
+    const GemmPlan p = plan_split(kEpiStoreF16, w_rows, M, split_k, split_k);
     if (p.splits == 1 && M > 64) continue;
     counters = std::max(counters, static_cast<size_t>(p.tok_tiles) * p.feat_tiles);
     if (p.splits > 1 && !gemm_cluster_ok(p.bn, p.splits))
@@ -1703,7 +1703,7 @@ int gs_linear(const void* x, const void* w, void* y, int M, int N, int K, int ep
   // split-K as the decoder plans it: across the CTAs of a cluster, through global
   // scratch (up to 64 rows), or as chunks inside each CTA
   const int w_rows = epilogue == kEpiSwiGLU ? 2 * N : N;
-  const GemmPlan p = plan_split(w_rows, M, split_k, K / 64);
+  const GemmPlan p = plan_split(epilogue, w_rows, M, split_k, K / 64);
   const int bn = p.bn, tok_tiles = p.tok_tiles, feat_tiles = p.feat_tiles;
   CUtensorMap tw, tx;
   if (!(epilogue == kEpiSwiGLU ? make_map_swiglu(&tw, w, N, K) : make_map(&tw, w, w_rows, K, 128)))

@@ -25,12 +25,12 @@ static cudaError_t launch_one(const CUtensorMap& tmW, const CUtensorMap& tmX, Ge
   // programmatic dependent launch.  Wider launches stream K through each CTA: the
   // deepest pipeline that still fits the CTAs one SM holds (one when the grid
   // is at most one CTA per SM, else two), since bytes in flight per SM set
-  // their load rate.  Clusters always two: with one CTA per SM a cluster of 8
+  // their load rate; the same for unsplit launches.  Clusters always two: with one CTA per SM a cluster of 8
   // waits for 8 empty SMs of one GPC (1024 x 4096 weight, 68 rows, 128 CTAs:
   // 17.4 us in the decoder's graph, 13.3 with two).
   const bool cl = a.splits > 1 && a.cluster;
   int want = S::kStagesDefault;
-  if (a.M > 64)
+  if (a.M > 64 || a.splits == 1)
     want = S::stages_fitting(
         !cl && static_cast<long>(feat_tiles) * tok_tiles * a.splits <= kNumSMs ? 1 : 2, EPI, cl);
   const int kb = a.kb_per_split;
@@ -63,7 +63,9 @@ static cudaError_t launch_bn(int epi, const CUtensorMap& tmW, const CUtensorMap&
 cudaError_t launch_gemm(int bn, int epi, const CUtensorMap& tmW, const CUtensorMap& tmX,
                         const GemmArgs& a, int feat_tiles, int tok_tiles, cudaStream_t s,
                         bool pdl) {
-  if (a.splits == 1) return launch_gemm_wide(bn, epi, tmW, tmX, a, feat_tiles, tok_tiles, s, pdl);
+  static_assert(kEpiQKVKind == kEpiQKV, "the dispatch rule's name for it");
+  if (a.splits == 1 && (a.chunks > 1 || !cta_per_tile(epi, feat_tiles, a.M, a.K / 64)))
+    return launch_gemm_wide(bn, epi, tmW, tmX, a, feat_tiles, tok_tiles, s, pdl);
   switch (bn) {
     case 32: return launch_bn<32>(epi, tmW, tmX, a, feat_tiles, tok_tiles, s, pdl);
     case 64: return launch_bn<64>(epi, tmW, tmX, a, feat_tiles, tok_tiles, s, pdl);

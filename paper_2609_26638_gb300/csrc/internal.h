@@ -42,6 +42,7 @@ cudaError_t launch_ex(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sm
 // SMs of one GB300 (two dies x 76).  Work decompositions that must not depend
 // on the device (the split-K factors) use this constant, not a query.
 constexpr int kNumSMs = 152;
+constexpr int kEpiQKVKind = 4;   // GemmEpilogue's kEpiQKV
 
 // Token tile of a GEMM over T token rows that splits K across CTAs.
 inline int gemm_bn_for(int T) { return T <= 32 ? 32 : (T <= 64 ? 64 : (T <= 128 ? 128 : 256)); }
@@ -68,9 +69,13 @@ constexpr int kWideTiles = 6;
 constexpr int kWideBN[kWideTiles] = {32, 64, 96, 144, 192, 256};
 constexpr int kWideCycles[kWideTiles] = {240, 257, 290, 350, 410, 515};
 
-inline int wide_index(int bn) {
-  for (int i = 0; i < kWideTiles; ++i)
-    if (kWideBN[i] == bn) return i;
+// The decoder's token maps: one per tile of either kernel.
+constexpr int kTokenMaps = kWideTiles + 1;
+constexpr int kTokenMapBN[kTokenMaps] = {32, 64, 96, 144, 192, 256, 128};
+
+inline int token_map_index(int bn) {
+  for (int i = 0; i < kTokenMaps; ++i)
+    if (kTokenMapBN[i] == bn) return i;
   return -1;
 }
 
@@ -98,6 +103,25 @@ inline int wide_bn(int feat_tiles, int T, int nkb) {
     }
   }
   return best;
+}
+
+// Unsplit launches of a little more than one wave of long tiles, one token tile:
+// the persistent kernel's one CTA per SM takes a second round of tiles on a few SMs,
+// where a CTA per tile, two on an SM, all start together (gemm_tc_kernel).
+// Measured, persistent / CTA per tile: 154 feature tiles x K 4096 34.7 / 29.8 us at
+// 17 rows, 39.8 / 32.1 at 64, 42.6 / 35.3 at 128; 190 x 8192 66.7 / 64.0, 77.9 / 68.3,
+// 81.5 / 72.6; 216 x 1024 14.4 / 13.3, 16.5 / 14.4, 18.9 / 17.0; even at 250, slower
+// at 152 and from 304 on.  193-256 rows, whose 256-row tiles have the shorter ring
+// beside the epilogue's slices, from K 8192 on and up to two tiles per SM: 154
+// feature tiles 109 / 93, 290 120 / 114 (at K 4096 48.9 / 51.6).
+inline bool cta_per_tile(int epi, int feat_tiles, int T, int nkb) {
+  if (feat_tiles <= kNumSMs) return false;
+  if (T <= (epi == kEpiQKVKind ? 64 : 128)) return 2 * feat_tiles <= 3 * kNumSMs;
+  return epi != kEpiQKVKind && T > 192 && T <= 256 && nkb >= 128 && feat_tiles <= 2 * kNumSMs;
+}
+// Token tile of a launch that does not split K across CTAs.
+inline int unsplit_bn(int epi, int feat_tiles, int T, int nkb, int chunks) {
+  return chunks <= 1 && cta_per_tile(epi, feat_tiles, T, nkb) ? gemm_bn_for(T) : wide_bn(feat_tiles, T, nkb);
 }
 
 cudaError_t launch_gemm(int bn, int epi, const CUtensorMap& tmW, const CUtensorMap& tmX,

@@ -78,8 +78,8 @@ extern "C" int gs_linear_noalloc(const void* x, const void* w, void* y, int M, i
   void* base = nullptr;
   int rc = scratch_for_current_device(&base);
   if (rc != GS_OK) return rc;
-  // unsplit launches run on the persistent kernel's token tiles
-  const int run_bn = split_k == 1 ? wide_bn(feat_tiles, M, K / 64) : bn;
+  // unsplit launches choose their own token tiles
+  const int run_bn = split_k == 1 ? unsplit_bn(epilogue, feat_tiles, M, K / 64, 1) : bn;
   const int run_tok_tiles = (M + run_bn - 1) / run_bn;
   CUtensorMap tw, tx;
   if (!(epilogue == kEpiSwiGLU ? make_map_swiglu(&tw, w, N, K) : make_map(&tw, w, w_rows, K, 128)))

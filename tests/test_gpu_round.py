@@ -436,3 +436,25 @@ def test_wide_model_batch_equals_single():
     slots = torch.arange(B, dtype=torch.int32, device=eng.device)
     assert decode_all(eng, slots, K, 40) == single
     eng.close()
+
+
+def test_weights_of_a_little_more_than_one_wave():
+    """Gate/up (160 tiles) and LM head (153 tiles) of one to one and a half tiles per
+    SM: one sequence in lock-step with the oracle (17-row windows), and a batch of
+    five (85 rows) commits what each commits alone."""
+    cfg = synth.TINY.with_(n_layers=1, n_heads=8, n_kv_heads=4, d_ffn=10240, vocab=153 * 128)
+    w = synth.make_weights(cfg, seed=17)
+    K, B, cap = 16, 5, 24
+    eng = new_engine(cfg, w, max_batch=B, max_ctx=256, max_K=K, max_prefill=128)
+    prompts = [synth.make_prompt(cfg, 20 + 9 * i, 5, index=80 + i) for i in range(B)]
+    st, stats = lockstep(eng, Decoder(cfg, w), prompts[0], K, cap, check_logits=True)
+    assert st.done
+    single = []
+    for i, p in enumerate(prompts):
+        eng.prefill(i, p.vis, p.text, cap)
+        single.append(decode_all(eng, torch.tensor([i], dtype=torch.int32, device=eng.device), K, 40)[0])
+    for i, p in enumerate(prompts):
+        eng.prefill(i, p.vis, p.text, cap)
+    slots = torch.arange(B, dtype=torch.int32, device=eng.device)
+    assert decode_all(eng, slots, K, 40) == single
+    eng.close()

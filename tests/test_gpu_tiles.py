@@ -288,3 +288,35 @@ def test_split_sums_through_scratch(gs, N, K, split, epi):
         gs.gs_linear_noalloc(xm.data_ptr(), w.data_ptr(), y.data_ptr(), M, N, K, epi, split, stream)
         assert gs.gs_linear_noalloc_status(stream) == gs.GS_OK
         assert torch.equal(y, want[:M]), M
+
+
+@pytest.mark.parametrize("tiles,K,Ms", [
+    (153, 256, (1, 32, 33, 64, 65, 128, 129)), (228, 192, (17, 64, 100, 128)), (229, 192, (17, 64, 128)),
+    (160, 8192, (40, 192, 193, 256, 257)),
+])
+@pytest.mark.parametrize("epi", [0, 1, 2, 3])
+def test_one_to_two_tiles_per_sm(gs, tiles, K, Ms, epi):
+    """Unsplit launches of a little more than one wave, on both sides of the sizes up
+    to which they take a CTA per tile: a row's bits are those of the 300-row window
+    (the persistent kernel), and the fp32 matmul is near."""
+    N = tiles * 64 if epi == gs.EPI_SWIGLU else tiles * 128
+    g = torch.Generator(device=DEV).manual_seed(tiles + epi)
+    x = torch.randn(300, K, device=DEV, generator=g).half()
+    w = (0.02 * torch.randn(tiles * 128, K, device=DEV, generator=g)).half()
+    base = torch.randn(300, N, device=DEV, generator=g)
+
+    def out(m):
+        if epi == gs.EPI_RESID_F32:
+            return base[:m].clone()
+        return (torch.zeros(m, dtype=torch.int64, device=DEV) if epi == gs.EPI_ARGMAX
+                else torch.zeros(m, N, dtype=torch.float16, device=DEV))
+
+    want = out(300)
+    _linear(gs, x, w, 300, N, K, epi, 1, want)
+    for M in Ms:
+        y = out(M)
+        _linear(gs, x[:M].contiguous(), w, M, N, K, epi, 1, y)
+        assert torch.equal(y, want[:M]), M
+    if epi == gs.EPI_STORE_F16:
+        ref = x.float() @ w.float().T
+        torch.testing.assert_close(want.float(), ref, rtol=2e-3, atol=1e-3 * ref.abs().max().item())
