@@ -182,17 +182,18 @@ int decode_splits(int weight_rows, int K) {
 // does every launch that is not split.  The sums and their order are the same.
 // Above 64 rows the persistent kernel's time is one tile's serial K, whatever the
 // rows: clusters of 8 with 64-token tiles keep the launches whose CTAs all fit
-// (two per SM) and have at least 8 k-blocks each.  us per launch, cluster /
+// (two per SM) and have at least 8 k-blocks each, clusters of 4 those of one per SM.  us per launch, cluster /
 // persistent, as graph nodes: 1024 x 4096 weight 9.4 / 14.1 at 65 rows, 10.7 /
 // 14.2 at 256 (256 CTAs), 15.0 / 14.3 at 320 (320 CTAs), 20.7 / 14.5 at 544;
 // 2048 x 8192 13.4 / 22.0 at 65, 21.0 / 21.9 at 129; 256 x 4096 7.2 / 13.3 at 65,
-// 9.5 / 14.1 at 544.  Clusters of 4 stay below one wave's worth of gain (4096 x
-// 2048: 11.3 / 9.9 at 128 rows, 4096 x 4096 14.1 / 14.0).
+// 9.5 / 14.1 at 544.  Clusters of 4: 1024 x 4096 11.5 / 13.9 (64-128 CTAs), 2048 x
+// 2048 9.5 / 10.0 at 128 CTAs and 10.8 / 10.2 at 192.
 GemmPlan plan_split(int epi, int weight_rows, int T, int S, int nkb) {
   GemmPlan p;
   p.feat_tiles = weight_rows / 128;
-  const bool clusters = S == kMaxClusterSplits && nkb / S >= 8 &&
-                        static_cast<long long>(p.feat_tiles) * cdiv(T, 64) * S <= 2 * kNumSMs;
+  const int per_sm = S == kMaxClusterSplits ? 2 : (S == 4 ? 1 : 0);
+  const bool clusters = nkb / S >= 8 &&
+                        static_cast<long long>(p.feat_tiles) * cdiv(T, 64) * S <= per_sm * kNumSMs;
   if (S > 1 && (T <= 64 || clusters)) {
     p.splits = S;
     p.chunks = 1;

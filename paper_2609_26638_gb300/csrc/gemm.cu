@@ -63,7 +63,8 @@ static cudaError_t launch_bn(int epi, const CUtensorMap& tmW, const CUtensorMap&
 cudaError_t launch_gemm(int bn, int epi, const CUtensorMap& tmW, const CUtensorMap& tmX,
                         const GemmArgs& a, int feat_tiles, int tok_tiles, cudaStream_t s,
                         bool pdl) {
-  static_assert(kEpiQKVKind == kEpiQKV, "the dispatch rule's name for it");
+  static_assert(kEpiStoreF16 == 0 && kEpiResidF32 == 1 && kEpiSwiGLUKind == kEpiSwiGLU && kEpiArgmax == 3 &&
+                    kEpiQKVKind == kEpiQKV, "the dispatch rules' names");
   if (a.splits == 1 && (a.chunks > 1 || !cta_per_tile(epi, feat_tiles, a.M, a.K / 64)))
     return launch_gemm_wide(bn, epi, tmW, tmX, a, feat_tiles, tok_tiles, s, pdl);
   switch (bn) {

@@ -27,9 +27,10 @@
 // shared epilogue on 32-token slices of it, while the MMAs of the next tile
 // fill the other buffers.
 //
-// What bounds it: the ring (measured per 64-deep k-block with one CTA per SM:
-// 240 / 257 cycles at BN 32 / 64, two k-blocks per stage, about 100 bytes per
-// clock and SM from L2; 350 at 144; 515 at 256, which is the MMA rate).  One
+// What bounds it: the ring.  Per 64-deep k-block, all 152 SMs running (K 8192 less K
+// 2048): 253 cycles at BN 32, 80 bytes per clock and SM from L2; 310 at 64 under
+// SwiGLU, 397 under the epilogues whose fp32 slices leave a stage less; 417 at 96; 435
+// / 460 at 144; 545 / 630 at 192; 720 / 840 at 256, where the MMA rate is 515.  One
 // CTA per tile instead paid its start-up, its first load latency and its
 // epilogue per tile: 544 rows of gate/up took 24.5 us, LM head at 17 rows 30 us,
 // a 4096-row prefill gate/up 100 us; here 19.0, 26.6 (23.6 as a graph node, 76% of

@@ -42,7 +42,8 @@ cudaError_t launch_ex(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sm
 // SMs of one GB300 (two dies x 76).  Work decompositions that must not depend
 // on the device (the split-K factors) use this constant, not a query.
 constexpr int kNumSMs = 152;
-constexpr int kEpiQKVKind = 4;   // GemmEpilogue's kEpiQKV
+// GemmEpilogue's values, for the dispatch rules.
+constexpr int kEpiSwiGLUKind = 2, kEpiQKVKind = 4;
 
 // Token tile of a GEMM over T token rows that splits K across CTAs.
 inline int gemm_bn_for(int T) { return T <= 32 ? 32 : (T <= 64 ? 64 : (T <= 128 ? 128 : 256)); }
@@ -61,13 +62,9 @@ inline bool gemm_cluster_ok(int bn, int splits) {
   const int per = bn / splits;
   return per <= 8 || 32 % per == 0;
 }
-// Token tiles of the persistent GEMM (splits == 1) and, per 64-deep k-block of
-// one, the cycles its ring takes with one CTA per SM (measured: 240 / 257 / 290
-// cycles at 32 / 64 / 96 rows, where L2 -> shared memory bounds it, 350 / 410 /
-// 515 at 144 / 192 / 256, towards the MMA rate of 2 cycles per row).
+// Token tiles of the persistent GEMM (splits == 1).
 constexpr int kWideTiles = 6;
 constexpr int kWideBN[kWideTiles] = {32, 64, 96, 144, 192, 256};
-constexpr int kWideCycles[kWideTiles] = {240, 257, 290, 350, 410, 515};
 
 // The decoder's token maps: one per tile of either kernel.
 constexpr int kTokenMaps = kWideTiles + 1;
@@ -79,24 +76,34 @@ inline int token_map_index(int bn) {
   return -1;
 }
 
-// The token tile with the least estimated time: rounds of tiles over the SMs,
-// each the longer of its k-blocks and its epilogue slices (about 2,000 cycles
-// per 32 tokens of a group; one group of warps at 32 rows, else two), and the
-// last tile's epilogue, which nothing overlaps.  The wider on a tie.  The slices'
-// cost is SwiGLU's.  Every tile measured at 128, 264, 544 and 1088 rows: the choice
-// is the fastest for O and down (residual) and within 3% of it for gate/up; for QKV's
-// shape with fp16 stores up to 544 rows too, but at 1088 its 64-row tiles take 13.4
-// us where 144 take 11.5 (such slices cost less than the rule counts).
-inline int wide_bn(int feat_tiles, int T, int nkb) {
+// The token tile with the least estimated time: rounds of tiles over the SMs, each a
+// start, its k-blocks and its epilogue, which share the SM (the longer and 0.63 of the
+// shorter).  The wider on a tie.  Cycles, fitted to 950 launches of every tile (four
+// epilogues, 68-4,096 rows, 256-59,392 features, K 64-8,192, 1-8 chunks): the choice
+// is 0.2% from the fastest tile in the mean and 8% at worst; one k-block and one
+// slice cost for all epilogues, made from long SwiGLU launches, was 3% and 121%
+// (fp16 stores of 4,096 x 16,384, K 448: 154 us with 64-row tiles, 70 with 256).
+// SwiGLU's fp16 slices leave the ring a stage more than the others' fp32 ones; a
+// chunk of an odd number of k-blocks fills half of a stage of two (32-96 rows); the
+// epilogue warps add up each chunk.
+inline int wide_bn(int epi, int feat_tiles, int T, int nkb, int chunks) {
+  constexpr double kBlock[2][kWideTiles] = {{207, 315, 388, 387, 586, 779}, {317, 394, 585, 611, 778, 1025}};
+  constexpr double kEpilogue[5][kWideTiles] = {{229, 1581, 1946, 3891, 5282, 8176},       // fp16 stores
+                                               {705, 2131, 6204, 10984, 14755, 25536},    // residual
+                                               {1185, 1350, 7219, 10301, 10664, 13872},   // SwiGLU
+                                               {1644, 1858, 6787, 10436, 11981, 17982},   // argmax
+                                               {229, 1581, 1946, 3891, 5282, 8176}};      // QKV, as stores
+  const int n = chunks > 1 ? chunks : 1;
+  const bool odd = nkb / n % 2 != 0;
   int best = 32;
-  long long best_cost = -1;
+  double best_cost = -1;
   for (int i = kWideTiles - 1; i >= 0; --i) {
     const int bn = kWideBN[i];
     const long long tiles = static_cast<long long>(feat_tiles) * ((T + bn - 1) / bn);
     const long long rounds = (tiles + kNumSMs - 1) / kNumSMs;
-    const long long main = static_cast<long long>(nkb) * kWideCycles[i];
-    const long long epi = 2000ll * ((bn / (bn >= 64 ? 2 : 1) + 31) / 32);
-    const long long cost = rounds * (main > epi ? main : epi) + epi;
+    const double main = nkb * kBlock[epi == kEpiSwiGLUKind][i] * (odd && bn <= 96 ? 1.38 : 1.0);
+    const double epilogue = kEpilogue[epi][i] + 0.7 * (n - 1) * bn;
+    const double cost = rounds * (main > epilogue ? main + 0.63 * epilogue + 3478 : epilogue + 0.63 * main + 3478);
     if (best_cost < 0 || cost < best_cost) {
       best_cost = cost;
       best = bn;
@@ -121,7 +128,7 @@ inline bool cta_per_tile(int epi, int feat_tiles, int T, int nkb) {
 }
 // Token tile of a launch that does not split K across CTAs.
 inline int unsplit_bn(int epi, int feat_tiles, int T, int nkb, int chunks) {
-  return chunks <= 1 && cta_per_tile(epi, feat_tiles, T, nkb) ? gemm_bn_for(T) : wide_bn(feat_tiles, T, nkb);
+  return chunks <= 1 && cta_per_tile(epi, feat_tiles, T, nkb) ? gemm_bn_for(T) : wide_bn(epi, feat_tiles, T, nkb, chunks);
 }
 
 cudaError_t launch_gemm(int bn, int epi, const CUtensorMap& tmW, const CUtensorMap& tmX,
