@@ -39,10 +39,14 @@ static cudaError_t launch_one(const CUtensorMap& tmW, const CUtensorMap& tmX, Ge
   const size_t smem = S::smem_bytes(a.stages, EPI, cl);
   if constexpr (S::kClusterOk) {
     if (cl)
-      return launch_ex(gemm_tc_kernel<BN, EPI, true>, grid, dim3(128), smem, s, pdl, dim3(1, 1, a.splits), tmW,
-                       tmX, a);
+      return launch_ex(gemm_tc_kernel<BN, EPI, kTcCluster>, grid, dim3(128), smem, s, pdl, dim3(1, 1, a.splits),
+                       tmW, tmX, a);
   }
-  return launch_ex(gemm_tc_kernel<BN, EPI, false>, grid, dim3(128), smem, s, pdl, dim3(1, 1, 1), tmW, tmX, a);
+  if (a.splits == 1)
+    return launch_ex(gemm_tc_kernel<BN, EPI, kTcWhole>, grid, dim3(128), smem, s, pdl, dim3(1, 1, 1), tmW, tmX,
+                     a);
+  return launch_ex(gemm_tc_kernel<BN, EPI, kTcScratch>, grid, dim3(128), smem, s, pdl, dim3(1, 1, 1), tmW, tmX,
+                   a);
 }
 
 template <int BN>
@@ -78,13 +82,18 @@ cudaError_t launch_gemm(int bn, int epi, const CUtensorMap& tmW, const CUtensorM
 
 template <int BN, int EPI>
 static cudaError_t set_attr_one() {
+  constexpr int bytes = GemmShape<BN>::kSmemMax;
   cudaError_t e = cudaSuccess;
   if constexpr (GemmShape<BN>::kClusterOk)
-    e = cudaFuncSetAttribute(gemm_tc_kernel<BN, EPI, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             GemmShape<BN>::kSmemMax);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(gemm_tc_kernel<BN, EPI, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              GemmShape<BN>::kSmemMax);
+    e = cudaFuncSetAttribute(gemm_tc_kernel<BN, EPI, kTcCluster>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             bytes);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(gemm_tc_kernel<BN, EPI, kTcWhole>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             bytes);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(gemm_tc_kernel<BN, EPI, kTcScratch>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             bytes);
+  return e;
 }
 
 template <int BN>
