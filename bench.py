@@ -69,14 +69,14 @@ def schedule_rounds(sched: np.ndarray, max_new: int) -> int:
 # traffic grows with the keys read: K and V rows, once each).
 _CSRC = os.path.join(ROOT, "paper_2609_26638_gb300", "csrc")
 NCU_TRAFFIC = {
-    "attention_b1": dict(sources=("attention.cuh", "ptx.cuh"), bytes=4934144, algorithmic=4823040,
-                         sha256="fcf89da96323a3a2d00a94b413726e715cbc6066eaf67e9db2f40475c1fab9a4"),
+    "attention_b1": dict(sources=("attention.cuh", "ptx.cuh"), bytes=4933632, algorithmic=4823040,
+                         sha256="e65de3d7b63efd06d9d6984b6aa82e2dd8481705471a2a2002241c30f4383728"),
     "attention_serve": dict(sources=("attention.cuh", "attention_stream.cuh", "ptx.cuh"),
-                            bytes=233444352, algorithmic=225173504,
-                            sha256="fc17e03133f39c4609f54fbf998e3f918ea503e4d84ec63e708dc39ecaa6ba7d"),
+                            bytes=231786496, algorithmic=225173504,
+                            sha256="f3b3eb736484f751e8d41c87b46f8492f503c306811aba686f8af7bb565a8952"),
     "lm_head_b1": dict(sources=("gemm_tc.cuh", "gemm_wide.cuh", "gemm_wide.cu", "ptx.cuh"),
-                       bytes=124607744, algorithmic=121669768,
-                       sha256="eabd23cf7a5c44b0d6dee526756fe7a54220d3439125dd7d591f85f4695422c3"),
+                       bytes=124707328, algorithmic=121669768,
+                       sha256="ea219724317878c6024d3baaa9aa436100edac7cee915bde8d246ec3b006bb01"),
 }
 
 
